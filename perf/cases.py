@@ -45,7 +45,7 @@ def listed():
         # one pass over a file larger than the cache, large pages: the benchmark's shape
         dict(scan, name="stream_1g", size=GiB, page=512 * KiB, cache=384 * MiB, stride=MiB, blocks=296),
         # the same with the paper's page size
-        dict(scan, name="stream_4k_pages", size=512 * MiB, page=4 * KiB, cache=64 * MiB, stride=MiB, blocks=296),
+        dict(scan, name="stream_4k_pages", size=GiB, page=4 * KiB, cache=256 * MiB, stride=MiB, blocks=296),
         # a file that the GPU cannot map (cold or direct files): host threads pread, the GPU copies
         dict(scan, name="stream_staged", size=256 * MiB, page=256 * KiB, cache=160 * MiB, stride=MiB, blocks=64,
              xfer=gfs.XFER_PULL),
@@ -232,8 +232,8 @@ class State:
 
 def prepare(case, seed):
     kind, page = case["kind"], case["page"]
-    # requests of up to a megabyte and readahead to match, as the benchmark configures them
-    cfg = dict(max_rpc_pages=min(256, max(16, MiB // page)), ra_cap_pages=min(255, max(8, 256 * KiB // page - 1)))
+    # request and readahead sizes as the benchmark configures them: 16 pages of the large sizes, 64 of the small
+    cfg = dict(max_rpc_pages=min(64, max(16, MiB // page)), ra_cap_pages=min(63, max(8, 256 * KiB // page - 1)))
     s = State(case, mode=case.get("mode", gfs.MODE_READAHEAD), xfer=case.get("xfer", gfs.XFER_MAPPED), **cfg)
     if kind == "serve":
         for i, n in enumerate(_file_sizes(case, seed)):
