@@ -38,7 +38,9 @@ __global__ void __launch_bounds__(kThreads) k_rowdot(DevHandle g, int fid, uint3
     for (uint32_t pr = r0; pr < r1; pr += rows_per_piece) {
       const uint32_t nr = pr + rows_per_piece < r1 ? rows_per_piece : r1 - pr;
       const unsigned long long off = (unsigned long long)pr * row_bytes;
-      const long long n = dev::gread_impl<true>(g, (int)blockIdx.x, fid, off, nr * row_bytes, buf, acc);
+      dev::BufferSink<true> sink{buf, off, acc};
+      const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, off, nr * row_bytes, sink);
+      acc = sink.acc;
       if (n != (long long)(nr * row_bytes)) {
         err = n < 0 ? n : -5;
         break;
@@ -105,7 +107,9 @@ __global__ void __launch_bounds__(kThreads) k_histogram(DevHandle g, int fid, un
   unsigned long long bad = 0;
   for (unsigned long long pc = blockIdx.x; pc < npieces; pc += gridDim.x) {
     const unsigned long long off = pc * read_len;
-    const long long n = dev::gread_impl<true>(g, (int)blockIdx.x, fid, off, read_len, buf, acc);
+    dev::BufferSink<true> sink{buf, off, acc};
+    const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, off, read_len, sink);
+    acc = sink.acc;
     if (n < 0) {
       if (threadIdx.x == 0) atomicCAS((unsigned long long*)status, 0ull, (unsigned long long)n);
       break;

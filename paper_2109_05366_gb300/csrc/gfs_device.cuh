@@ -2005,22 +2005,26 @@ static __device__ void release_page(const DevHandle& g, int f, uint32_t nbytes, 
 }
 
 // ---------------------------------------------------------------- page runs
-// With small pages a page's control chain (lookup, pin, mark check, release)
-// costs more than its copy, so a gread takes up to 32 consecutive pages that are
-// already in the cache at once, one lane per page.  A run ends before the first
-// page that is missing, in error, being reclaimed, or READY with a readahead
-// mark still set (R4 stays with the one-page path, at the page's turn).  The
-// pages of a run are released in page order, so the consumed FIFO receives the
-// same pushes, in the same order, as from pages read one at a time.
-constexpr uint32_t kRunMaxShift = 14;  // runs for pages of at most 16 KiB
-constexpr uint32_t kRunPages = 32;
+// A page's control chain (lookup, pin, state, mark check, release) is a string of
+// L2 round trips that costs a block 4 to 5 us, whatever the page's size.  A gread
+// therefore takes the consecutive pages that are already in the cache at once, one
+// lane per page and 32 pages per warp, every warp of the block: up to kRunPages
+// pages share one chain.  A run ends before the first page that is missing, in
+// error, being reclaimed, or READY with a readahead mark still set (R4 stays with
+// the one-page path, at the page's turn).  The pages of a run are released in page
+// order, so the consumed FIFO receives the same pushes, in the same order, as from
+// pages read one at a time.
+// Bound by latency: 257 cached greads of 1 MiB in 4 KiB pages by 256-thread blocks took
+// 257 us with one warp looking up 32 pages a run, 120 us with all eight.
+constexpr uint32_t kRunWarps = 16;  // warps that look pages up (the widest block of the library's own kernels)
+constexpr uint32_t kRunPages = 32 * kRunWarps;
 
-// Warp 0: look up and pin pages p .. p + k - 1 (k <= 32).  Returns the length of
+// Warp: look up and pin pages p .. p + k - 1 (k <= 32).  Returns the length of
 // the leading run of pages that are READY without a mark, FILLING or COPYING;
-// their frames and states are left in s_f / s_st, pinned.  Pages after the run
-// are left unpinned.
+// their frames are left in s_f, pinned, and the mask of those not READY yet in
+// *wait.  Pages after the run are left unpinned.
 static __device__ uint32_t run_begin(const DevHandle& g, uint32_t fid, unsigned long long p, uint32_t k, bool marks,
-                                     uint32_t* s_f, int* s_st) {
+                                     uint32_t* s_f, uint32_t* wait) {
   const int lane = lane_id();
   int f = -1;  // frame of page p + lane
   // home buckets only, eight keys in flight: a key in an overflow bucket ends the run
@@ -2057,43 +2061,68 @@ static __device__ uint32_t run_begin(const DevHandle& g, uint32_t fid, unsigned 
   const unsigned okm = __ballot_sync(kFull, ok);
   const uint32_t c = okm == kFull ? 32u : (uint32_t)(__ffs(~okm) - 1);
   if (mine && (uint32_t)lane >= c) atomicSub(&g.fpins[f], 1u);
-  if ((uint32_t)lane < c) {
-    s_f[lane] = (uint32_t)f;
-    s_st[lane] = st;
-  }
+  const unsigned wm = __ballot_sync(kFull, (uint32_t)lane < c && st != FR_READY);
+  if ((uint32_t)lane < c) s_f[lane] = (uint32_t)f;
+  if (lane == 0) *wait = wm;
   __syncwarp();
   return c;
 }
 
-// Warp 0, after the block copied the run: R5 for its n pages (page p + i in frame
-// s_f[i]; the gread covers [off, end)).  FIFO cells are reserved with one ticket
-// add and filled in page order.
+// One lane, one page of a run (frame f, page q; the gread covers [off, end)): R5's
+// accounting.  Returns whether the page goes to the consumed FIFO.
+static __device__ bool run_consume(const DevHandle& g, uint32_t f, unsigned long long q, unsigned long long off,
+                                   unsigned long long end) {
+  const unsigned long long base = q << g.page_shift;
+  const unsigned long long lo = off > base ? off : base;
+  const unsigned long long hi = end < base + g.page_size ? end : base + g.page_size;
+  const uint32_t nb = (uint32_t)(hi - lo);
+  const uint32_t c = atomicAdd(&g.fconsumed[f], nb);
+  if (g.repl == GFS_REPL_TB_LRA) return false;  // per-threadblock LRA queues keep no consumed FIFO
+  const uint32_t v = ld_rlx(&g.fvalid[f]);
+  return c < v && c + nb >= v;
+}
+
+// Whole block, after it read the run: R5 for its n pages (page p + i in frame
+// s_f[i]; the gread covers [off, end)), a lane per page, the warps that looked them
+// up.  FIFO cells are reserved with one ticket add for the run and filled in page
+// order.
 static __device__ void run_release(const DevHandle& g, const uint32_t* s_f, uint32_t n, unsigned long long p,
                                    unsigned long long off, unsigned long long end, unsigned long long deadline) {
-  const int lane = lane_id();
-  const bool mine = (uint32_t)lane < n;
-  bool push = false;
-  uint32_t f = 0;
-  if (mine) {
-    f = s_f[lane];
-    const unsigned long long base = (p + lane) << g.page_shift;
-    const unsigned long long lo = off > base ? off : base;
-    const unsigned long long hi = end < base + g.page_size ? end : base + g.page_size;
-    const uint32_t nb = (uint32_t)(hi - lo);
-    const uint32_t c = atomicAdd(&g.fconsumed[f], nb);
-    if (g.repl != GFS_REPL_TB_LRA) {  // per-threadblock LRA queues keep no consumed FIFO
-      const uint32_t v = ld_rlx(&g.fvalid[f]);
-      push = c < v && c + nb >= v;
-    }
-  }
+  __shared__ uint32_t s_push[kRunWarps];
+  __shared__ unsigned long long s_t0;
+  const uint32_t tid = threadIdx.x, w = tid >> 5, lane = tid & 31u;
+  if (n <= 32 && w) return;  // one warp's run: no block-wide step
+  const bool mine = tid < n;
+  const uint32_t f = mine ? s_f[tid] : 0u;
+  const bool push = mine && run_consume(g, f, p + tid, off, end);
   __threadfence();
   if (mine) atomicSub(&g.fpins[f], 1u);
-  const unsigned m = __ballot_sync(kFull, push);
-  if (!m) return;
-  unsigned long long t0 = 0;
-  if (lane == 0) t0 = atomicAdd(&g.ctrl->fifo_tail.v, (unsigned long long)__popc(m));
-  t0 = bcast64(t0);
-  if (push) fifo_put(g, t0 + (unsigned long long)__popc(m & ((1u << lane) - 1u)), f, deadline);
+  unsigned m;
+  unsigned long long t = 0;
+  if (n <= 32) {
+    m = __ballot_sync(kFull, push);
+    if (!m) return;
+    if (lane == 0) t = atomicAdd(&g.ctrl->fifo_tail.v, (unsigned long long)__popc(m));
+    t = bcast64(t);
+  } else {
+    if (!__syncthreads_or(push)) return;
+    m = 0;
+    if (32 * w < n) {  // whole warps
+      m = __ballot_sync(kFull, push);
+      if (lane == 0) s_push[w] = (uint32_t)__popc(m);
+    }
+    __syncthreads();
+    const uint32_t nrw = (n + 31) >> 5;
+    if (tid == 0) {
+      uint32_t all = 0;
+      for (uint32_t i = 0; i < nrw; ++i) all += s_push[i];
+      s_t0 = atomicAdd(&g.ctrl->fifo_tail.v, (unsigned long long)all);
+    }
+    __syncthreads();
+    t = s_t0;
+    for (uint32_t i = 0; i < w && i < nrw; ++i) t += s_push[i];
+  }
+  if (push) fifo_put(g, t + (unsigned long long)__popc(m & ((1u << lane) - 1u)), f, deadline);
   __syncwarp();
 }
 
@@ -2134,97 +2163,85 @@ __device__ __forceinline__ uint4 shift16(const uint4& a, const uint4& b, uint32_
                     __funnelshift_r(w3, w4, r8));
 }
 
-// Copy n bytes of a cache frame (src) to the user buffer (dst), thread `tid` of
-// the `nt` that share the copy (whole warps; all their lanes call it).  Frame data
-// is read through L2 (ld.global.cg): frames are rewritten by the copy engine, so L1
-// may hold an older page.  With FUSED the checksums of the copied bytes are
-// accumulated on the way (src_off = file offset of src[0]).
-// Bound by the loads in flight.  dst is brought to a 16-byte boundary by a head of
-// single bytes; the body is stored 16 bytes a thread.  Where src then sits at
-// another phase, a thread loads the aligned 16 bytes its chunk starts in, takes the
-// next 16 from its neighbour lane (lane 31 loads them) and shifts the two.  The
-// aligned words all hold at least one byte of the range, so nothing outside the
-// frame is read (frames start on a page boundary and are whole 16-byte words).
-// Measured on 16384 cached reads of 256 B .. 64 KiB at any byte (64 KiB pages): 159 us;
-// a byte a thread at unequal phases, as before: 1273 us (every 32-byte sector was
-// fetched again by each of the 32 single-byte loads).
+constexpr uint32_t kUnitShift = 12;  // a warp checksums 4 KiB at a time (pages are at least that large)
+constexpr uint32_t kCopyShift = 11;  // and copies 2 KiB at a time
+constexpr uint32_t kCopyWords = (1u << kCopyShift) / 16;
+
+// Warp: unit c of the copy of n bytes of a cache frame (src) to the user buffer
+// (dst): the 16-byte words 128 c .. 128 c + 127 of dst past its head of single bytes
+// (unit 0 also copies the head and the tail).  Frame data is read through L2
+// (ld.global.cg): frames are rewritten by the copy engine, so L1 may hold an older
+// page.  With FUSED the checksums of the copied bytes are accumulated on the way
+// (src_off = file offset of src[0]).
+// Bound by the loads in flight: a lane has the four 16-byte loads of its unit under way
+// before it stores.  Units of 2 KiB share a read of a few KiB among the warps of a block
+// and fit the 64-register instance: 16384 cached reads of 256 B .. 64 KiB, one by one,
+// take 211 us; units of 4 KiB took 233 us.
+// Where src sits at another phase of a 16-byte word than dst, a lane loads the
+// aligned word its chunk starts in, takes the next from its neighbour lane and
+// shifts the two.  The aligned words all hold at least one byte of the range, so
+// nothing outside the frame is read (frames start on a page boundary and are whole
+// 16-byte words).  The same reads took 1273 us a byte a thread.
 template <bool FUSED>
-__device__ __forceinline__ void copy_range(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, uint32_t n,
-                                           unsigned long long src_off, Sums& acc, uint32_t tid, uint32_t nt) {
+__device__ __forceinline__ void copy_unit(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, uint32_t n,
+                                          uint32_t c, unsigned long long src_off, Sums& acc) {
+  const uint32_t lane = threadIdx.x & 31u;
   uint32_t head = (16u - (uint32_t)((uintptr_t)dst & 15)) & 15u;
   if (head > n) head = n;
   const uint32_t n16 = (n - head) >> 4, tail = head + 16 * n16;
-  // at most 15 head bytes and 15 tail bytes, in one pass of 32 threads
-  if (tid < 32 && (head | (n - tail))) {
-    const uint32_t j = tid < 16 ? tid : tail + (tid - 16);
-    if (tid < 16 ? j < head : j < n) {
+  if (c == 0 && (head | (n - tail))) {  // at most 15 head bytes and 15 tail bytes
+    const uint32_t j = lane < 16 ? lane : tail + (lane - 16);
+    if (lane < 16 ? j < head : j < n) {
       const uint8_t b = __ldcg(src + j);
       dst[j] = b;
       if (FUSED) sums_add1(acc, b, src_off + j);
     }
   }
-  uint4* d4 = reinterpret_cast<uint4*>(dst + head);
-  const unsigned long long o0 = src_off + head;
+  const uint32_t i0 = c * kCopyWords;
+  if (i0 >= n16) return;
+  uint4* d4 = reinterpret_cast<uint4*>(dst + head) + i0 + lane;
+  const uint32_t left = n16 - i0;  // words from this unit on
   const uint32_t sh = (uint32_t)((uintptr_t)(src + head) & 15);
+  const uint4* w4 = reinterpret_cast<const uint4*>(src + head - sh) + i0 + lane;
+  const unsigned long long o = src_off + head + 16ull * (i0 + lane);
+  uint4 v[4];
   if (sh == 0) {
-    const uint4* s4 = reinterpret_cast<const uint4*>(src + head);
-    uint32_t i = tid;
-    for (; i + 3 * nt < n16; i += 4 * nt) {
-      uint4 a = __ldcg(s4 + i), b = __ldcg(s4 + i + nt), c = __ldcg(s4 + i + 2 * nt), d = __ldcg(s4 + i + 3 * nt);
-      d4[i] = a;
-      d4[i + nt] = b;
-      d4[i + 2 * nt] = c;
-      d4[i + 3 * nt] = d;
-      if (FUSED) {
-        const unsigned long long o = o0 + 16ull * i;
-        sums_add16(acc, a, o);
-        sums_add16(acc, b, o + 16ull * nt);
-        sums_add16(acc, c, o + 32ull * nt);
-        sums_add16(acc, d, o + 48ull * nt);
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u)
+      if (lane + 32 * u < left) v[u] = __ldcg(w4 + 32 * u);
+#pragma unroll
+    for (uint32_t u = 0; u < 4; ++u)
+      if (lane + 32 * u < left) {
+        d4[32 * u] = v[u];
+        if (FUSED) sums_add16(acc, v[u], o + 512 * u);
       }
-    }
-    for (; i < n16; i += nt) {
-      uint4 a = __ldcg(s4 + i);
-      d4[i] = a;
-      if (FUSED) sums_add16(acc, a, o0 + 16ull * i);
-    }
     return;
   }
-  const uint4* w4 = reinterpret_cast<const uint4*>(src + head - sh);  // words 0 .. n16
-  const uint32_t q = sh >> 2, r8 = 8 * (sh & 3), lane = tid & 31;
-  for (uint32_t base = tid - lane; base < n16; base += 4 * nt) {  // warp-uniform
-    uint4 v[4], x[4];
+  const uint32_t q = sh >> 2, r8 = 8 * (sh & 3);
+  uint4 x = make_uint4(0u, 0u, 0u, 0u);  // the word after the unit's last (lane 31 uses it)
 #pragma unroll
-    for (uint32_t u = 0; u < 4; ++u) {
-      const uint32_t i = base + u * nt + lane;
-      v[u] = x[u] = make_uint4(0u, 0u, 0u, 0u);
-      if (i <= n16) v[u] = __ldcg(w4 + i);
-      if (lane == 31 && i < n16) x[u] = __ldcg(w4 + i + 1);
-    }
+  for (uint32_t u = 0; u < 4; ++u) {
+    v[u] = make_uint4(0u, 0u, 0u, 0u);
+    if (lane + 32 * u <= left) v[u] = __ldcg(w4 + 32 * u);
+  }
+  if (lane == 31 && kCopyWords <= left) x = __ldcg(w4 + 97);
 #pragma unroll
-    for (uint32_t u = 0; u < 4; ++u) {
-      const uint32_t i = base + u * nt + lane;
-      uint4 y;
-      y.x = __shfl_down_sync(kFull, v[u].x, 1);
-      y.y = __shfl_down_sync(kFull, v[u].y, 1);
-      y.z = __shfl_down_sync(kFull, v[u].z, 1);
-      y.w = __shfl_down_sync(kFull, v[u].w, 1);
-      if (lane == 31) y = x[u];
-      if (i < n16) {
-        const uint4 a = shift16(v[u], y, q, r8);
-        d4[i] = a;
-        if (FUSED) sums_add16(acc, a, o0 + 16ull * i);
-      }
+  for (uint32_t u = 0; u < 4; ++u) {
+    // lane 31's next word is lane 0's of the following 32
+    const uint4 z = u < 3 ? v[u < 3 ? u + 1 : 3] : make_uint4(0u, 0u, 0u, 0u);
+    const bool first = lane == 0;
+    uint4 y;
+    y.x = __shfl_sync(kFull, first ? z.x : v[u].x, lane + 1);
+    y.y = __shfl_sync(kFull, first ? z.y : v[u].y, lane + 1);
+    y.z = __shfl_sync(kFull, first ? z.z : v[u].z, lane + 1);
+    y.w = __shfl_sync(kFull, first ? z.w : v[u].w, lane + 1);
+    if (u == 3 && lane == 31) y = x;
+    if (lane + 32 * u < left) {
+      y = shift16(v[u], y, q, r8);
+      d4[32 * u] = y;
+      if (FUSED) sums_add16(acc, y, o + 512 * u);
     }
   }
-}
-
-// The whole block copies (its whole warps, where its size is no multiple of 32).
-template <bool FUSED>
-__device__ __forceinline__ void copy_out(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, uint32_t n,
-                                         unsigned long long src_off, Sums& acc) {
-  const uint32_t nt = blockDim.x & ~31u;
-  if (threadIdx.x < nt) copy_range<FUSED>(src, dst, n, src_off, acc, threadIdx.x, nt);
 }
 
 // Block-wide sum of two u64 values (mod 2^64); the result is valid in thread 0.
@@ -2252,80 +2269,128 @@ __device__ __forceinline__ void block_sum2(unsigned long long& a, unsigned long 
 }
 
 // ---------------------------------------------------------------- gread
-// Whole block: read the run of cached pages that starts at page p (p1 = last
-// page of the gread, which covers [off, end) into buf): pin it, wait for pages
-// still being filled in page order, copy it a warp per page, release it.  Returns
-// the number of pages read (0: page p takes the one-page path) or -errno.
-// Kept out of line so that it leaves the one-page path's registers alone.
+// Bytes [lo, hi) of a file whose pages p, p + 1, ... are pinned, READY, in the frames
+// f[0], f[1], ... (f in shared memory): what a gread hands its sink, piece by piece in
+// file order.  Sink::take(g, r) is called by the whole block; the pages stay pinned
+// until every thread has returned from it.
+struct RunView {
+  const uint32_t* f;
+  unsigned long long p, lo, hi;
+};
+// The frame byte of offset `rel` counted from the start of page r.p.
+__device__ __forceinline__ const uint8_t* run_at(const DevHandle& g, const RunView& r, unsigned long long rel) {
+  return g.frames + ((size_t)r.f[rel >> g.page_shift] << g.page_shift) + ((uint32_t)rel & (g.page_size - 1u));
+}
+
+// The gread into a user buffer: the byte at offset off goes to buf[0].  A warp takes a
+// unit of a page at a time.  With FUSED the checksums of the bytes go to acc.
 template <bool FUSED>
+struct BufferSink {
+  uint8_t* buf;
+  unsigned long long off;
+  Sums acc;
+  __device__ __noinline__ void take(const DevHandle& g, const RunView& r) {
+    const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (w >= nw) return;  // the last lanes of a block that is no multiple of 32
+    Sums part{0ull, 0ull};
+    const uint32_t ush = g.page_shift - kCopyShift, last = (uint32_t)(((r.hi - 1) >> g.page_shift) - r.p);
+    for (uint32_t u = w; u < (last + 1) << ush; u += nw) {
+      const uint32_t j = u >> ush;
+      const unsigned long long base = (r.p + j) << g.page_shift;
+      const uint32_t lo = j == 0 ? (uint32_t)(r.lo - base) : 0u;
+      const uint32_t hi = j == last ? (uint32_t)(r.hi - base) : g.page_size;
+      copy_unit<FUSED>(g.frames + ((size_t)r.f[j] << g.page_shift) + lo, buf + (base + lo - off), hi - lo,
+                       u & ((1u << ush) - 1u), base + lo, part);
+    }
+    if (FUSED) {
+      acc.sum += part.sum;
+      acc.hash += part.hash;
+    }
+  }
+};
+
+// Whole block: read the run of cached pages that starts at page p (p1 = last
+// page of the gread, which covers [off, end)): pin it, wait for pages still being
+// filled in page order, hand it to the sink, release it.  Returns the number of
+// pages read (0: page p takes the one-page path) or -errno.
+// Kept out of line so that it leaves the one-page path's registers alone.
+template <class Sink>
 __device__ __noinline__ long long read_run(const DevHandle& g, uint32_t fid, unsigned long long p,
                                            unsigned long long p1, unsigned long long off, unsigned long long end,
-                                           uint8_t* buf, bool marks, unsigned long long deadline, Sums* part) {
-  __shared__ uint32_t s_rf[kRunPages], s_rn;
-  __shared__ int s_rst[kRunPages], s_mark;
-  const uint32_t tid = threadIdx.x;
-  if (tid < 32) {
-    const unsigned long long left = p1 - p + 1;
-    const uint32_t c = run_begin(g, fid, p, left < kRunPages ? (uint32_t)left : kRunPages, marks, s_rf, s_rst);
-    if (tid == 0) s_rn = c;
+                                           Sink& sink, bool marks, unsigned long long deadline) {
+  __shared__ uint32_t s_rf[kRunPages], s_rn[kRunWarps], s_rwait[kRunWarps];
+  __shared__ int s_mark;
+  const uint32_t tid = threadIdx.x, w = tid >> 5;
+  const uint32_t nw = (blockDim.x >> 5) < kRunWarps ? blockDim.x >> 5 : kRunWarps;
+  const unsigned long long left = p1 - p + 1;
+  const uint32_t want = left < 32u * nw ? (uint32_t)left : 32u * nw;  // pages looked up
+  uint32_t c = 0;                                                   // this warp's leading pages
+  if (32 * w < want) {
+    c = run_begin(g, fid, p + 32 * w, want - 32 * w < 32 ? want - 32 * w : 32, marks, s_rf + 32 * w, &s_rwait[w]);
+    if ((tid & 31) == 0) s_rn[w] = c;
   }
   __syncthreads();
-  uint32_t n = s_rn;
+  uint32_t n = 0, rw = 0;  // the run; the warps that hold it
+  while (32 * rw < want) {
+    n += s_rn[rw];
+    if (s_rn[rw++] < 32) break;
+  }
+  if (w >= rw && (tid & 31) < c) atomicSub(&g.fpins[s_rf[tid]], 1u);  // pages past the first gap
   // a mark found on a waited page once it is READY ends the run before it
-  for (uint32_t i = 0; i < n; ++i) {
-    if (s_rst[i] == FR_READY) continue;
-    const int st = block_wait_ready(g, (int)s_rf[i], deadline);
-    if (st != FR_READY) {
-      if (tid == 0) {
-        for (uint32_t j = 0; j < n; ++j) frame_unpin(g, (int)s_rf[j]);
-        stat_add(g, ST_HITS, i + 1);
-        if (st == FR_ERROR) stat_add(g, ST_EIO, 1);
+  uint32_t waited = 0;
+  for (uint32_t v = 0; v < rw; ++v) {
+    for (uint32_t m = s_rwait[v]; m; m &= m - 1) {
+      const uint32_t i = 32 * v + (uint32_t)(__ffs(m) - 1);
+      if (i >= n) break;
+      const int st = block_wait_ready(g, (int)s_rf[i], deadline);
+      if (st != FR_READY) {
+        if (tid == 0) {
+          for (uint32_t j = 0; j < n; ++j) frame_unpin(g, (int)s_rf[j]);
+          stat_add(g, ST_HITS, i + 1);
+          if (st == FR_ERROR) stat_add(g, ST_EIO, 1);
+        }
+        __syncthreads();
+        return st < 0 ? st : -kEIO;
       }
-      __syncthreads();
-      return st < 0 ? st : -kEIO;
-    }
-    if (marks) {
-      if (tid == 0) s_mark = ld_rlx(&g.fmark[s_rf[i]]) != 0u;
-      __syncthreads();
-      const int mk = s_mark;
-      __syncthreads();
-      if (mk) {
-        if (tid == 0)
-          for (uint32_t j = i; j < n; ++j) frame_unpin(g, (int)s_rf[j]);
-        n = i;
+      if (marks) {
+        if (tid == 0) s_mark = ld_rlx(&g.fmark[s_rf[i]]) != 0u;
+        __syncthreads();
+        const int mk = s_mark;
+        __syncthreads();
+        if (mk) {
+          if (tid == 0)
+            for (uint32_t j = i; j < n; ++j) frame_unpin(g, (int)s_rf[j]);
+          n = i;
+          break;
+        }
       }
+      ++waited;
     }
   }
-  if (n == 0) return 0;
+  if (n == 0) {
+    __syncthreads();
+    return 0;
+  }
   if (tid == 0) {
-    uint32_t waited = 0;
-    for (uint32_t i = 0; i < n; ++i) waited += s_rst[i] != FR_READY;
     stat_add(g, ST_HITS, n);
     stat_add(g, ST_COALESCED, waited);
   }
-  Sums acc{0ull, 0ull};
-  const uint32_t lane = tid & 31, nw = blockDim.x >> 5;
-  for (uint32_t i = tid >> 5; i < n && (tid >> 5) < nw; i += nw) {  // a whole warp per page
-    const unsigned long long base = (p + i) << g.page_shift;
-    const unsigned long long lo = (off > base ? off : base) - base;
-    const unsigned long long hi = (end < base + g.page_size ? end : base + g.page_size) - base;
-    copy_range<FUSED>(g.frames + ((size_t)s_rf[i] << g.page_shift) + lo, buf + (base + lo - off),
-                      (uint32_t)(hi - lo), base + lo, acc, lane, 32);
-  }
-  if (FUSED) *part = acc;
+  const unsigned long long base = p << g.page_shift, lim = (p + n) << g.page_shift;
+  sink.take(g, RunView{s_rf, p, off > base ? off : base, end < lim ? end : lim});
   __syncthreads();
-  if (tid < 32) run_release(g, s_rf, n, p, off, end, deadline);
+  run_release(g, s_rf, n, p, off, end, deadline);
   return n;
 }
 
-// Threadblock-collective read of [off, off + len) of file `fid` into buf.
+// Threadblock-collective read of [off, off + len) of file `fid` into a sink.
 // Every thread of the block must call it with the same arguments.  `stream`
 // identifies the reader for sequential detection (the threadblock).  Returns
 // the byte count (short at EOF, 0 at or past EOF) or a negative errno.
-template <bool FUSED>
+template <class Sink>
 __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigned long long off,
-                                unsigned long long len, uint8_t* buf, Sums& acc) {
+                                unsigned long long len, Sink& sink) {
   __shared__ int s_frame, s_state;
+  __shared__ uint32_t s_one;
   __shared__ unsigned long long s_seq0;
   __shared__ PaperJob s_job;
   __shared__ uint32_t s_frames[MAX_RPC_PAGES];
@@ -2342,21 +2407,16 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
   const unsigned long long seq0 = s_seq0;
   const unsigned long long deadline = now_ns() + g.timeout_ns;
   long long err = 0;
-  const bool runs = g.mode != GFS_MODE_PAPER && g.page_shift <= kRunMaxShift && p1 > p0;
+  const bool runs = g.mode != GFS_MODE_PAPER && p1 > p0;
   const bool marks = g.mode == GFS_MODE_READAHEAD && g.async_ra && fi.ra;
   for (unsigned long long p = p0; p <= p1;) {
     if (runs) {
-      Sums part{0ull, 0ull};
-      const long long n = read_run<FUSED>(g, (uint32_t)fid, p, p1, off, end, buf, marks, deadline, &part);
+      const long long n = read_run(g, (uint32_t)fid, p, p1, off, end, sink, marks, deadline);
       if (n < 0) {
         err = n;
         break;
       }
       if (n) {
-        if (FUSED) {
-          acc.sum += part.sum;
-          acc.hash += part.hash;
-        }
         p += (unsigned long long)n;
         continue;
       }
@@ -2371,6 +2431,7 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
       int r = acquire_begin(g, stream, (uint32_t)fid, fi, p, p1, seq0, deadline, s_frames, &st, &s_job);
       if (tid == 0) {
         s_frame = r;
+        s_one = (uint32_t)r;
         s_state = st;
       }
     }
@@ -2399,10 +2460,9 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
     __syncthreads();
     block_self_serve(g, fi, s_frames);  // the asynchronous window check_mark requested, if any
     const unsigned long long base = p << g.page_shift;
-    const unsigned long long lo = (off > base ? off : base) - base;
-    const unsigned long long hi = (end < base + g.page_size ? end : base + g.page_size) - base;
-    copy_out<FUSED>(g.frames + ((size_t)f << g.page_shift) + lo, buf + (base + lo - off), (uint32_t)(hi - lo),
-                    base + lo, acc);
+    const unsigned long long lo = off > base ? off : base;
+    const unsigned long long hi = end < base + g.page_size ? end : base + g.page_size;
+    sink.take(g, RunView{&s_one, p, lo, hi});
     __syncthreads();
     if (tid == 0) release_page(g, f, (uint32_t)(hi - lo), deadline);
     ++p;
@@ -2419,8 +2479,8 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
 
 __device__ __forceinline__ long long gread(const DevHandle& g, int stream, int fid, unsigned long long off,
                                            unsigned long long len, void* buf) {
-  Sums unused{0, 0};
-  return gread_impl<false>(g, stream, fid, off, len, (uint8_t*)buf, unused);
+  BufferSink<false> sink{(uint8_t*)buf, off, {0ull, 0ull}};
+  return gread_impl(g, stream, fid, off, len, sink);
 }
 
 // File size of an open fid, or -EBADF.  Any thread.

@@ -26,8 +26,9 @@ __global__ void __launch_bounds__(512, 1) k_scan_path(DevHandle g, const __grid_
   const int fid = dev::gopen(g, path.s, GFS_RDONLY);
   const long long size = fid >= 0 ? dev::gfstat_size(g, fid) : (long long)fid;
   for (unsigned long long s = b; s < nstrides; s += gridDim.x) {
-    Sums acc{0ull, 0ull};
-    const long long r = size < 0 ? size : dev::gread_impl<true>(g, (int)b, fid, s * stride, read_len, buf, acc);
+    dev::BufferSink<true> sink{buf, s * stride, {0ull, 0ull}};
+    const long long r = size < 0 ? size : dev::gread_impl(g, (int)b, fid, s * stride, read_len, sink);
+    Sums acc = sink.acc;
     dev::block_sum2(acc.sum, acc.hash);
     if (tid == 0) {
       cnt[s] = r;

@@ -86,8 +86,9 @@ __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsig
       }
       __syncthreads();
     }
-    Sums acc{0ull, 0ull};
-    long long r = dev::gread_impl<FUSED>(g, (int)b, fid, off, read_len, buf, acc);
+    dev::BufferSink<FUSED> sink{buf, off, {0ull, 0ull}};
+    long long r = dev::gread_impl(g, (int)b, fid, off, read_len, sink);
+    Sums acc = sink.acc;
     if (serialize) {  // wait until every request of this gread has been served
       block_quiesce(g);
       if (tid == 0) dev::st_rel64(&g.ctrl->ticket.v, s + 1);

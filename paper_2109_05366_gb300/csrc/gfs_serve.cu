@@ -242,8 +242,9 @@ __global__ void __launch_bounds__(512) k_serve(DevHandle g, Handle h) {
       continue;
     }
     idle_ns = 256;
-    dev::Sums acc{0ull, 0ull};
-    const long long n = dev::gread_impl<true>(g, (int)blockIdx.x, (int)s_fid, s_off, s_len, buf, acc);
+    dev::BufferSink<true> sink{buf, s_off, {0ull, 0ull}};
+    const long long n = dev::gread_impl(g, (int)blockIdx.x, (int)s_fid, s_off, s_len, sink);
+    dev::Sums acc = sink.acc;
     dev::block_sum2(acc.sum, acc.hash);
     if (tid == 0) {
       Req& q = h.req[r];
