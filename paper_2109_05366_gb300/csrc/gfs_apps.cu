@@ -4,8 +4,9 @@
 //                  per-row dot products with a resident vector;
 //   gfs_histogram  an int32 array streamed into a histogram.
 // Both gread their input in read_len pieces through the page cache, so every
-// byte they consume came through the same path as the stride scan; both also
-// report checksums of the bytes they consumed.
+// byte they consume came through the same path as the stride scan, and consume
+// it where its pages lie (their sinks copy nothing); both also report checksums
+// of the bytes they consumed.
 #include <cuda_runtime.h>
 #include <errno.h>
 
@@ -18,50 +19,162 @@ namespace {
 constexpr uint32_t kThreads = 256;
 constexpr uint32_t kSmemBins = 8192;  // histogram bins kept in shared memory (the heavy head of a Zipf law)
 
+// Dot products of the rows of one gread (off: its first byte, whole rows) taken where
+// their pages lie in the cache.  A warp takes consecutive rows, four at a time where
+// they share a page, so that each load of the vector serves four rows; lane l takes the
+// float4 columns l, l + 32, ... of a row in that order, whatever the pages.  A row cut
+// by the end of a run of pages leaves its lanes' partial sums in `carry`, from where the
+// next run goes on with them.
+// Bound by HBM reads and the loads in flight.  Rows read from a gread buffer crossed HBM
+// three times (out of the cache, into the buffer, back in): a cached 16384 x 8192 matrix
+// took 303 us that way and takes 135 us in place.
+struct RowdotSink {
+  const float4* vec;
+  float* out;  // the gread's first row
+  float4* carry;  // shared memory, 2 x 32; one half is read while the other is written
+  unsigned long long off, row_bytes;
+  uint32_t cols4, half;
+  dev::Sums acc;
+
+  // R whole rows that follow each other from p on (file offset o), all in one page.
+  template <int R>
+  __device__ __forceinline__ void rows_in_page(const uint8_t* p, unsigned long long o, uint32_t row,
+                                               dev::Sums& part) const {
+    constexpr int U = 8 / R;
+    const uint32_t lane = threadIdx.x & 31u;
+    float4 s[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) s[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t c = lane;
+    for (; c + 32 * (U - 1) < cols4; c += 32 * U) {
+      uint4 x[R][U];
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          x[i][u] = __ldcg(reinterpret_cast<const uint4*>(p + (size_t)i * row_bytes) + c + 32 * u);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float4 y = __ldg(vec + c + 32 * u);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          fma4(s[i], x[i][u], y);
+          dev::sums_add16(part, x[i][u], o + (unsigned long long)i * row_bytes + 16ull * (c + 32 * u));
+        }
+      }
+    }
+    for (; c < cols4; c += 32) {
+      const float4 y = __ldg(vec + c);
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const uint4 x = __ldcg(reinterpret_cast<const uint4*>(p + (size_t)i * row_bytes) + c);
+        fma4(s[i], x, y);
+        dev::sums_add16(part, x, o + (unsigned long long)i * row_bytes + 16ull * c);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) finish(s[i], row + (uint32_t)i);
+  }
+
+  // The part of row `row` that the view holds; pages may change inside it.
+  __device__ __forceinline__ void row_any(const DevHandle& g, const dev::RunView& r, uint32_t row, dev::Sums& part) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const unsigned long long o = off + row * row_bytes, base = r.p << g.page_shift;
+    const uint32_t c0 = r.lo > o ? (uint32_t)((r.lo - o) >> 4) : 0u;
+    const uint32_t c1 = r.hi < o + row_bytes ? (uint32_t)((r.hi - o) >> 4) : cols4;
+    float4 s = c0 ? carry[32 * half + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t c = c0 <= lane ? lane : lane + ((c0 - lane + 31u) & ~31u);
+    for (; c < c1; c += 32 * 8) {
+      uint4 x[8];
+#pragma unroll
+      for (uint32_t u = 0; u < 8; ++u)
+        if (c + 32 * u < c1)
+          x[u] = __ldcg(reinterpret_cast<const uint4*>(dev::run_at(g, r, o + 16ull * (c + 32 * u) - base)));
+#pragma unroll
+      for (uint32_t u = 0; u < 8; ++u)
+        if (c + 32 * u < c1) {
+          fma4(s, x[u], __ldg(vec + c + 32 * u));
+          dev::sums_add16(part, x[u], o + 16ull * (c + 32 * u));
+        }
+    }
+    if (c1 < cols4) carry[32 * (half ^ 1u) + lane] = s;
+    else finish(s, row);
+  }
+
+  static __device__ __forceinline__ void fma4(float4& s, const uint4& x, const float4& y) {
+    s.x = fmaf(__uint_as_float(x.x), y.x, s.x);
+    s.y = fmaf(__uint_as_float(x.y), y.y, s.y);
+    s.z = fmaf(__uint_as_float(x.z), y.z, s.z);
+    s.w = fmaf(__uint_as_float(x.w), y.w, s.w);
+  }
+  __device__ __forceinline__ void finish(const float4& v, uint32_t row) const {
+    float s = (v.x + v.y) + (v.z + v.w);
+    for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(dev::kFull, s, d);
+    if ((threadIdx.x & 31) == 0) out[row] = s;
+  }
+
+  __device__ __noinline__ void take(const DevHandle& g, const dev::RunView& r) {
+    const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const uint32_t first = (uint32_t)((r.lo - off) / row_bytes), last = (uint32_t)((r.hi - 1 - off) / row_bytes);
+    const uint32_t per = (last - first + nw) / nw;  // rows a warp
+    uint32_t row = first + w * per;
+    const uint32_t stop = row + per < last + 1 ? row + per : last + 1;
+    const unsigned long long base = r.p << g.page_shift;
+    dev::Sums part{0ull, 0ull};
+    while (row < stop) {
+      const unsigned long long o = off + row * row_bytes;
+      // whole rows from this one on that end before its page does
+      uint32_t k = 0;
+      if (o >= r.lo) {
+        const unsigned long long page_end = (o | (g.page_size - 1u)) + 1;
+        const unsigned long long lim = page_end < r.hi ? page_end : r.hi;
+        while (k < 4 && row + k < stop && o + (k + 1) * row_bytes <= lim) ++k;
+      }
+      if (k == 0) {
+        row_any(g, r, row, part);
+        ++row;
+        continue;
+      }
+      const uint8_t* p = dev::run_at(g, r, o - base);
+      if (k == 4) rows_in_page<4>(p, o, row, part);
+      else if (k >= 2) rows_in_page<2>(p, o, row, part);
+      else rows_in_page<1>(p, o, row, part);
+      row += k == 4 ? 4 : (k >= 2 ? 2 : 1);
+    }
+    half ^= 1u;
+    acc.sum += part.sum;
+    acc.hash += part.hash;
+  }
+};
+
 // Block b reads stripes b, b + B, ...; a stripe is `stripe_rows` rows and is read
-// in pieces of `read_len` bytes (whole rows).  Each warp takes rows of the piece.
+// in pieces of `read_len` bytes (whole rows).
 __global__ void __launch_bounds__(kThreads) k_rowdot(DevHandle g, int fid, uint32_t rows, uint32_t cols,
                                                      const float* __restrict__ vec, float* __restrict__ out,
-                                                     uint32_t stripe_rows, unsigned long long read_len, uint8_t* bufs,
-                                                     unsigned long long buf_stride, unsigned long long* stripe_sum,
+                                                     uint32_t stripe_rows, unsigned long long read_len,
+                                                     unsigned long long* stripe_sum,
                                                      unsigned long long* stripe_hash, long long* status) {
-  uint8_t* buf = bufs + (size_t)blockIdx.x * buf_stride;
+  __shared__ float4 s_carry[64];
   const unsigned long long row_bytes = (unsigned long long)cols * 4;
   const uint32_t rows_per_piece = (uint32_t)(read_len / row_bytes);
   const uint32_t nstripes = (rows + stripe_rows - 1) / stripe_rows;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  RowdotSink sink{reinterpret_cast<const float4*>(vec), out, s_carry, 0ull, row_bytes, cols / 4, 0u, {0ull, 0ull}};
   for (uint32_t st = blockIdx.x; st < nstripes; st += gridDim.x) {
     const uint32_t r0 = st * stripe_rows;
     const uint32_t r1 = r0 + stripe_rows < rows ? r0 + stripe_rows : rows;
-    dev::Sums acc{0ull, 0ull};
+    sink.acc = dev::Sums{0ull, 0ull};
     long long err = 0;
     for (uint32_t pr = r0; pr < r1; pr += rows_per_piece) {
       const uint32_t nr = pr + rows_per_piece < r1 ? rows_per_piece : r1 - pr;
-      const unsigned long long off = (unsigned long long)pr * row_bytes;
-      dev::BufferSink<true> sink{buf, off, acc};
-      const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, off, nr * row_bytes, sink);
-      acc = sink.acc;
+      sink.off = (unsigned long long)pr * row_bytes;
+      sink.out = out + pr;
+      const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, sink.off, nr * row_bytes, sink);
       if (n != (long long)(nr * row_bytes)) {
         err = n < 0 ? n : -5;
         break;
       }
-      for (uint32_t r = warp; r < nr; r += nwarps) {
-        const float4* a = reinterpret_cast<const float4*>(buf + (size_t)r * row_bytes);
-        const float4* v = reinterpret_cast<const float4*>(vec);
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        for (uint32_t c = lane; c < cols / 4; c += 32) {
-          const float4 x = a[c], y = __ldg(v + c);
-          s0 = fmaf(x.x, y.x, s0);
-          s1 = fmaf(x.y, y.y, s1);
-          s2 = fmaf(x.z, y.z, s2);
-          s3 = fmaf(x.w, y.w, s3);
-        }
-        float s = (s0 + s1) + (s2 + s3);
-        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(dev::kFull, s, o);
-        if (lane == 0) out[pr + r] = s;
-      }
-      __syncthreads();
     }
+    dev::Sums acc = sink.acc;
     dev::block_sum2(acc.sum, acc.hash);
     if (threadIdx.x == 0) {
       stripe_sum[st] = acc.sum;
@@ -75,79 +188,76 @@ __global__ void __launch_bounds__(kThreads) k_rowdot(DevHandle g, int fid, uint3
       if (!dev::block_help(g, -1, true)) break;
 }
 
-// One value of the histogram (warp-collective: every lane calls it, `have` says
-// whether the lane holds a value).  Bins below kSmemBins go to shared memory; the
-// rest to global memory, lanes holding the same value adding once; values at or
-// above nbins are counted in `bad`.
-__device__ __forceinline__ void count_value(uint32_t* sh, uint32_t* hist, uint32_t nbins, uint32_t v, bool have,
-                                            unsigned long long& bad) {
-  if (have && v < kSmemBins && v < nbins) atomicAdd(&sh[v], 1u);
-  if (have && v >= nbins) ++bad;
-  const bool far = have && v >= kSmemBins && v < nbins;
-  const unsigned fm = __ballot_sync(dev::kFull, far);
-  if (far) {
-    const unsigned same = __match_any_sync(fm, v);
-    if ((threadIdx.x & 31) == (uint32_t)(__ffs(same) - 1)) atomicAdd(&hist[v], (uint32_t)__popc(same));
+// Counts the int32 values of a gread that starts at a multiple of 16, where their pages
+// lie in the cache.  Bins below kSmemBins (the heavy head of a Zipf law) are counted in
+// shared memory, the rest with one global atomic a value: they repeat too seldom within
+// a warp for a match among its lanes to pay.  (First pass over 256 MiB: 1746 us with a
+// buffer and the match, 1602 us without; 1280 us is the host link.)  A last value of fewer
+// than four bytes is not counted.
+struct HistSink {
+  uint32_t* sh;
+  uint32_t* hist;
+  uint32_t nbins;
+  unsigned long long bad;
+  dev::Sums acc;
+  __device__ __forceinline__ void count(uint32_t v) {
+    if (v >= nbins) ++bad;
+    else if (v < kSmemBins) atomicAdd(&sh[v], 1u);
+    else atomicAdd(&hist[v], 1u);
   }
-}
+  __device__ __noinline__ void take(const DevHandle& g, const dev::RunView& r) {
+    const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31u, units = dev::run_units(r);
+    const unsigned long long end = r.hi & ~3ull;
+    dev::Sums part{0ull, 0ull};
+    for (uint32_t u = w; u < units; u += nw) {
+      const unsigned long long at = r.lo + ((unsigned long long)u << dev::kUnitShift);
+      uint4 v[8];
+      dev::load_unit(g, r, at, v);
+      dev::unit_sums(part, v, at);
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) {
+        const unsigned long long q = at + 16 * lane + 512 * k;
+        if (q + 16 <= end) {
+          count(v[k].x);
+          count(v[k].y);
+          count(v[k].z);
+          count(v[k].w);
+        } else {
+          if (q + 4 <= end) count(v[k].x);
+          if (q + 8 <= end) count(v[k].y);
+          if (q + 12 <= end) count(v[k].z);
+        }
+      }
+    }
+    acc.sum += part.sum;
+    acc.hash += part.hash;
+  }
+};
 
-// Block b reads pieces b, b + B, ... of the int32 file and counts values.  Bins
-// below kSmemBins are counted in shared memory; the rest with warp-aggregated
-// global atomics (lanes holding the same value add once).
+// Block b reads pieces b, b + B, ... of the int32 file and counts values.
 __global__ void __launch_bounds__(kThreads) k_histogram(DevHandle g, int fid, unsigned long long size, uint32_t nbins,
                                                         uint32_t* __restrict__ hist, unsigned long long read_len,
-                                                        uint8_t* bufs, unsigned long long buf_stride,
                                                         unsigned long long* sums, long long* status) {
   __shared__ uint32_t sh[kSmemBins];
   for (uint32_t i = threadIdx.x; i < kSmemBins; i += blockDim.x) sh[i] = 0;
   __syncthreads();
-  uint8_t* buf = bufs + (size_t)blockIdx.x * buf_stride;
   const unsigned long long npieces = (size + read_len - 1) / read_len;
-  dev::Sums acc{0ull, 0ull};
-  unsigned long long bad = 0;
+  HistSink sink{sh, hist, nbins, 0ull, {0ull, 0ull}};
   for (unsigned long long pc = blockIdx.x; pc < npieces; pc += gridDim.x) {
-    const unsigned long long off = pc * read_len;
-    dev::BufferSink<true> sink{buf, off, acc};
-    const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, off, read_len, sink);
-    acc = sink.acc;
+    const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, pc * read_len, read_len, sink);
     if (n < 0) {
       if (threadIdx.x == 0) atomicCAS((unsigned long long*)status, 0ull, (unsigned long long)n);
       break;
     }
-    const uint32_t nv = (uint32_t)(n / 4);
-    const uint32_t* vals = reinterpret_cast<const uint32_t*>(buf);
-    // 16-byte loads, two per thread in flight (the buffer is 256-byte aligned), then
-    // the values left over after the last whole 16 bytes one per thread; every
-    // trip count is block-uniform (the far-bin path is warp-collective)
-    const uint4* v4 = reinterpret_cast<const uint4*>(buf);
-    const uint32_t n4 = nv / 4, nt = blockDim.x;
-    for (uint32_t base = 0; base < n4; base += 2 * nt) {
-      const uint32_t i = base + threadIdx.x, j = i + nt;
-      const uint4 a = i < n4 ? v4[i] : make_uint4(0u, 0u, 0u, 0u);
-      const uint4 b = j < n4 ? v4[j] : make_uint4(0u, 0u, 0u, 0u);
-      count_value(sh, hist, nbins, a.x, i < n4, bad);
-      count_value(sh, hist, nbins, a.y, i < n4, bad);
-      count_value(sh, hist, nbins, a.z, i < n4, bad);
-      count_value(sh, hist, nbins, a.w, i < n4, bad);
-      count_value(sh, hist, nbins, b.x, j < n4, bad);
-      count_value(sh, hist, nbins, b.y, j < n4, bad);
-      count_value(sh, hist, nbins, b.z, j < n4, bad);
-      count_value(sh, hist, nbins, b.w, j < n4, bad);
-    }
-    for (uint32_t base = 4 * n4; base < nv; base += nt) {
-      const uint32_t i = base + threadIdx.x;
-      count_value(sh, hist, nbins, i < nv ? vals[i] : 0u, i < nv, bad);
-    }
-    __syncthreads();
   }
   __syncthreads();
   for (uint32_t i = threadIdx.x; i < kSmemBins && i < nbins; i += blockDim.x)
     if (sh[i]) atomicAdd(&hist[i], sh[i]);
-  unsigned long long b2 = bad;
-  dev::block_sum2(acc.sum, b2);
+  unsigned long long total = sink.acc.sum, bad = sink.bad;
+  dev::block_sum2(total, bad);
   if (threadIdx.x == 0) {
-    atomicAdd(&sums[0], acc.sum);
-    atomicAdd(&sums[1], b2);
+    atomicAdd(&sums[0], total);
+    atomicAdd(&sums[1], bad);
   }
   if (g.xfer != GFS_XFER_DMA)
     for (int i = 0; i < 4096; ++i)
@@ -168,18 +278,16 @@ extern "C" int gfs_rowdot(gfs_ctx* ctx, int fid, uint32_t rows, uint32_t cols, c
   const uint64_t row_bytes = (uint64_t)cols * 4;
   if (read_len < row_bytes || read_len % row_bytes) return -EINVAL;  // pieces of whole rows
   if ((uint64_t)rows * row_bytes > ctx->files[fid].size) return -EINVAL;
-  const uint64_t stride = (read_len + 255) / 256 * 256;
-  int rc = ensure_scan_buf(ctx, (size_t)blocks * stride);
-  if (!rc) rc = ensure_paper_state(ctx, blocks);
+  if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;
+  const int rc = ensure_paper_state(ctx, blocks);
   if (rc) return rc;
   DevHandle g = ctx->dev;
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
                                       : blocks * (uint32_t)((read_len + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(d_status, 0, 8, s) != cudaSuccess) return -EINVAL;
-  k_rowdot<<<blocks, kThreads, 0, s>>>(g, fid, rows, cols, d_vec, d_out, stripe_rows, read_len, ctx->d_scan_buf,
-                                       stride, (unsigned long long*)d_stripe_sum,
-                                       (unsigned long long*)d_stripe_hash, (long long*)d_status);
+  k_rowdot<<<blocks, kThreads, 0, s>>>(g, fid, rows, cols, d_vec, d_out, stripe_rows, read_len,
+                                       (unsigned long long*)d_stripe_sum, (unsigned long long*)d_stripe_hash, (long long*)d_status);
   return cudaGetLastError() == cudaSuccess ? 0 : -EINVAL;
 }
 
@@ -188,9 +296,8 @@ extern "C" int gfs_histogram(gfs_ctx* ctx, int fid, uint32_t nbins, uint32_t* d_
   if (!ctx || !d_hist || !d_sums || !d_status) return -EINVAL;
   if (fid < 0 || (size_t)fid >= ctx->files.size() || !ctx->files[fid].open) return -EBADF;
   if (nbins == 0 || read_len == 0 || read_len % 16 || blocks == 0) return -EINVAL;
-  const uint64_t stride = (read_len + 255) / 256 * 256;
-  int rc = ensure_scan_buf(ctx, (size_t)blocks * stride);
-  if (!rc) rc = ensure_paper_state(ctx, blocks);
+  if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;
+  const int rc = ensure_paper_state(ctx, blocks);
   if (rc) return rc;
   DevHandle g = ctx->dev;
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
@@ -199,7 +306,7 @@ extern "C" int gfs_histogram(gfs_ctx* ctx, int fid, uint32_t nbins, uint32_t* d_
   if (cudaMemsetAsync(d_hist, 0, (size_t)nbins * 4, s) != cudaSuccess) return -EINVAL;
   if (cudaMemsetAsync(d_sums, 0, 16, s) != cudaSuccess) return -EINVAL;
   if (cudaMemsetAsync(d_status, 0, 8, s) != cudaSuccess) return -EINVAL;
-  k_histogram<<<blocks, kThreads, 0, s>>>(g, fid, ctx->files[fid].size, nbins, d_hist, read_len, ctx->d_scan_buf,
-                                          stride, (unsigned long long*)d_sums, (long long*)d_status);
+  k_histogram<<<blocks, kThreads, 0, s>>>(g, fid, ctx->files[fid].size, nbins, d_hist, read_len,
+                                          (unsigned long long*)d_sums, (long long*)d_status);
   return cudaGetLastError() == cudaSuccess ? 0 : -EINVAL;
 }

@@ -10,9 +10,10 @@
 //                                                  work: CTAs pick active
 //                                                  requests round-robin and
 //                                                  claim one unit (a stride of
-//                                                  unit_bytes) at a time; gread
-//                                                  + checksum; per-request sums
-//                                                  add up (mod 2^64)
+//                                                  unit_bytes) at a time; gread,
+//                                                  checksummed in place;
+//                                                  per-request sums add up
+//                                                  (mod 2^64)
 //   gfs_poll        <- completion ring (mapped) <- the CTA finishing a
 //                                                  request's last unit
 //
@@ -72,8 +73,7 @@ struct Handle {
   Req* req;
   Ctl* ctl;
   const uint32_t* stop;  // mapped host flag
-  uint8_t* bufs;
-  unsigned long long unit_bytes, buf_stride, idle_exit_ns;
+  unsigned long long unit_bytes, idle_exit_ns;
   uint32_t sub_slots, compl_slots, max_req, units_cap, pages_per_unit, frame_budget;
 };
 
@@ -197,7 +197,6 @@ __global__ void __launch_bounds__(512) k_serve(DevHandle g, Handle h) {
   __shared__ unsigned long long s_off, s_len;
   __shared__ uint32_t s_fid;
   const uint32_t tid = threadIdx.x;
-  uint8_t* buf = h.bufs + (size_t)blockIdx.x * h.buf_stride;
   unsigned idle_ns = 256;
   for (;;) {
     if (tid == 0) {
@@ -242,7 +241,7 @@ __global__ void __launch_bounds__(512) k_serve(DevHandle g, Handle h) {
       continue;
     }
     idle_ns = 256;
-    dev::BufferSink<true> sink{buf, s_off, {0ull, 0ull}};
+    dev::SumSink sink{{0ull, 0ull}};
     const long long n = dev::gread_impl(g, (int)blockIdx.x, (int)s_fid, s_off, s_len, sink);
     dev::Sums acc = sink.acc;
     dev::block_sum2(acc.sum, acc.hash);
@@ -318,7 +317,6 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   h.compl_slots = sc->queue_slots;
   h.max_req = sc->max_requests;
   h.unit_bytes = sc->unit_bytes;
-  h.buf_stride = (sc->unit_bytes + 255) / 256 * 256;
   h.units_cap = sc->units_in_flight ? sc->units_in_flight : 16;
   h.pages_per_unit = (uint32_t)((sc->unit_bytes + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;
   const uint32_t F = ctx->dev.n_frames;
@@ -327,8 +325,7 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   h.idle_exit_ns = sc->idle_exit_ms ? (unsigned long long)sc->idle_exit_ms * 1000000ull : 60ull * 1000000000ull;
   const size_t req_bytes = sizeof(Req) * h.max_req;
   const size_t ctl_off = (req_bytes + 255) / 256 * 256;
-  const size_t buf_off = ctl_off + (sizeof(Ctl) + 255) / 256 * 256;
-  const size_t total = buf_off + (size_t)sc->ctas * h.buf_stride;
+  const size_t total = ctl_off + sizeof(Ctl);
   rc = cerr(cudaMalloc((void**)&s->d_mem, total));
   if (!rc) rc = cerr(cudaMemset(s->d_mem, 0, total));
   if (!rc) rc = cerr(cudaHostAlloc((void**)&s->h_sub, sizeof(SubSlot) * h.sub_slots, cudaHostAllocMapped));
@@ -352,7 +349,6 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   h.stop = (const uint32_t*)p;
   h.req = (Req*)s->d_mem;
   h.ctl = (Ctl*)(s->d_mem + ctl_off);
-  h.bufs = s->d_mem + buf_off;
   if (rc) {
     free_server(s);
     return rc;
