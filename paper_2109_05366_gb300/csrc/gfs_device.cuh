@@ -2171,8 +2171,7 @@ constexpr uint32_t kCopyWords = (1u << kCopyShift) / 16;
 // (dst): the 16-byte words 128 c .. 128 c + 127 of dst past its head of single bytes
 // (unit 0 also copies the head and the tail).  Frame data is read through L2
 // (ld.global.cg): frames are rewritten by the copy engine, so L1 may hold an older
-// page.  With FUSED the checksums of the copied bytes are accumulated on the way
-// (src_off = file offset of src[0]).
+// page.
 // Bound by the loads in flight: a lane has the four 16-byte loads of its unit under way
 // before it stores.  Units of 2 KiB share a read of a few KiB among the warps of a block
 // and fit the 64-register instance: 16384 cached reads of 256 B .. 64 KiB, one by one,
@@ -2182,20 +2181,15 @@ constexpr uint32_t kCopyWords = (1u << kCopyShift) / 16;
 // shifts the two.  The aligned words all hold at least one byte of the range, so
 // nothing outside the frame is read (frames start on a page boundary and are whole
 // 16-byte words).  The same reads took 1273 us a byte a thread.
-template <bool FUSED>
 __device__ __forceinline__ void copy_unit(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, uint32_t n,
-                                          uint32_t c, unsigned long long src_off, Sums& acc) {
+                                          uint32_t c) {
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t head = (16u - (uint32_t)((uintptr_t)dst & 15)) & 15u;
   if (head > n) head = n;
   const uint32_t n16 = (n - head) >> 4, tail = head + 16 * n16;
   if (c == 0 && (head | (n - tail))) {  // at most 15 head bytes and 15 tail bytes
     const uint32_t j = lane < 16 ? lane : tail + (lane - 16);
-    if (lane < 16 ? j < head : j < n) {
-      const uint8_t b = __ldcg(src + j);
-      dst[j] = b;
-      if (FUSED) sums_add1(acc, b, src_off + j);
-    }
+    if (lane < 16 ? j < head : j < n) dst[j] = __ldcg(src + j);
   }
   const uint32_t i0 = c * kCopyWords;
   if (i0 >= n16) return;
@@ -2203,7 +2197,6 @@ __device__ __forceinline__ void copy_unit(const uint8_t* __restrict__ src, uint8
   const uint32_t left = n16 - i0;  // words from this unit on
   const uint32_t sh = (uint32_t)((uintptr_t)(src + head) & 15);
   const uint4* w4 = reinterpret_cast<const uint4*>(src + head - sh) + i0 + lane;
-  const unsigned long long o = src_off + head + 16ull * (i0 + lane);
   uint4 v[4];
   if (sh == 0) {
 #pragma unroll
@@ -2211,10 +2204,7 @@ __device__ __forceinline__ void copy_unit(const uint8_t* __restrict__ src, uint8
       if (lane + 32 * u < left) v[u] = __ldcg(w4 + 32 * u);
 #pragma unroll
     for (uint32_t u = 0; u < 4; ++u)
-      if (lane + 32 * u < left) {
-        d4[32 * u] = v[u];
-        if (FUSED) sums_add16(acc, v[u], o + 512 * u);
-      }
+      if (lane + 32 * u < left) d4[32 * u] = v[u];
     return;
   }
   const uint32_t q = sh >> 2, r8 = 8 * (sh & 3);
@@ -2236,11 +2226,7 @@ __device__ __forceinline__ void copy_unit(const uint8_t* __restrict__ src, uint8
     y.z = __shfl_sync(kFull, first ? z.z : v[u].z, lane + 1);
     y.w = __shfl_sync(kFull, first ? z.w : v[u].w, lane + 1);
     if (u == 3 && lane == 31) y = x;
-    if (lane + 32 * u < left) {
-      y = shift16(v[u], y, q, r8);
-      d4[32 * u] = y;
-      if (FUSED) sums_add16(acc, y, o + 512 * u);
-    }
+    if (lane + 32 * u < left) d4[32 * u] = shift16(v[u], y, q, r8);
   }
 }
 
@@ -2283,28 +2269,21 @@ __device__ __forceinline__ const uint8_t* run_at(const DevHandle& g, const RunVi
 }
 
 // The gread into a user buffer: the byte at offset off goes to buf[0].  A warp takes a
-// unit of a page at a time.  With FUSED the checksums of the bytes go to acc.
-template <bool FUSED>
+// unit of a page at a time.
 struct BufferSink {
   uint8_t* buf;
   unsigned long long off;
-  Sums acc;
   __device__ __noinline__ void take(const DevHandle& g, const RunView& r) {
     const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (w >= nw) return;  // the last lanes of a block that is no multiple of 32
-    Sums part{0ull, 0ull};
     const uint32_t ush = g.page_shift - kCopyShift, last = (uint32_t)(((r.hi - 1) >> g.page_shift) - r.p);
     for (uint32_t u = w; u < (last + 1) << ush; u += nw) {
       const uint32_t j = u >> ush;
       const unsigned long long base = (r.p + j) << g.page_shift;
       const uint32_t lo = j == 0 ? (uint32_t)(r.lo - base) : 0u;
       const uint32_t hi = j == last ? (uint32_t)(r.hi - base) : g.page_size;
-      copy_unit<FUSED>(g.frames + ((size_t)r.f[j] << g.page_shift) + lo, buf + (base + lo - off), hi - lo,
-                       u & ((1u << ush) - 1u), base + lo, part);
-    }
-    if (FUSED) {
-      acc.sum += part.sum;
-      acc.hash += part.hash;
+      copy_unit(g.frames + ((size_t)r.f[j] << g.page_shift) + lo, buf + (base + lo - off), hi - lo,
+                u & ((1u << ush) - 1u));
     }
   }
 };
@@ -2392,6 +2371,55 @@ struct SumSink {
       uint4 v[8];
       load_unit(g, r, at, v);
       unit_sums(part, v, at);
+    }
+    acc.sum += part.sum;
+    acc.hash += part.hash;
+  }
+};
+
+// The stride scan's consumer: a gread delivered through a window of the block's
+// buffer, kScanUnits units for each warp, that is read back as it fills (FUSED:
+// checksummed on the way in instead, without the read back).
+// Bound by HBM: the window stays in L2 (296 blocks of 256 threads: 37 MiB), so a cached
+// byte moves over HBM once.  Buffers of a whole read (310 MB) did not: each byte was
+// read, written, evicted and read again.  A cached 1 GiB scan, 296 blocks, 512 KiB pages:
+// 579 us with whole buffers, 296 us with windows.
+// A warp reads back only what it delivered, so the block does not wait for itself;
+// unit u always goes to the same cell, by the same warp.
+constexpr uint32_t kScanUnits = SCAN_UNITS;
+static_assert(SCAN_UNIT_BYTES == 1u << kUnitShift, "a cell holds a unit");
+template <bool FUSED>
+struct ScanSink {
+  uint8_t* buf;  // scan_window() bytes, 16-byte aligned
+  Sums acc;
+  __device__ __noinline__ void take(const DevHandle& g, const RunView& r) {
+    const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31u, units = run_units(r);
+    const unsigned long long o = r.lo & ~15ull;
+    Sums part{0ull, 0ull};
+    for (uint32_t u0 = w; u0 < units; u0 += kScanUnits * nw) {
+#pragma unroll 1
+      for (uint32_t i = 0; i < kScanUnits && u0 + i * nw < units; ++i) {
+        const unsigned long long at = o + ((unsigned long long)(u0 + i * nw) << kUnitShift);
+        uint4* cell = reinterpret_cast<uint4*>(buf + ((size_t)(w + i * nw) << kUnitShift)) + lane;
+        uint4 v[8];
+        load_unit(g, r, at, v);
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k)
+          if (at + 16 * lane + 512 * k < r.hi) cell[32 * k] = v[k];
+        if (FUSED) unit_sums(part, v, at);
+      }
+      if (FUSED) continue;
+      __syncwarp();
+#pragma unroll 1
+      for (uint32_t i = 0; i < kScanUnits && u0 + i * nw < units; ++i) {
+        const unsigned long long at = o + ((unsigned long long)(u0 + i * nw) << kUnitShift);
+        const uint4* cell = reinterpret_cast<const uint4*>(buf + ((size_t)(w + i * nw) << kUnitShift)) + lane;
+        uint4 v[8];
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k)
+          v[k] = at + 16 * lane + 512 * k < r.hi ? cell[32 * k] : make_uint4(0u, 0u, 0u, 0u);
+        unit_sums(part, v, at);
+      }
     }
     acc.sum += part.sum;
     acc.hash += part.hash;
@@ -2568,7 +2596,7 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
 
 __device__ __forceinline__ long long gread(const DevHandle& g, int stream, int fid, unsigned long long off,
                                            unsigned long long len, void* buf) {
-  BufferSink<false> sink{(uint8_t*)buf, off, {0ull, 0ull}};
+  BufferSink sink{(uint8_t*)buf, off};
   return gread_impl(g, stream, fid, off, len, sink);
 }
 

@@ -1245,8 +1245,9 @@ static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t*
   // no size wraps around
   const uint64_t per_block = std::min<uint64_t>(a->read_len, size);
   if (per_block > SIZE_MAX / 2) return -ENOMEM;
-  *buf_stride = align_up(per_block, 256);
-  if (*buf_stride && a->blocks > SIZE_MAX / *buf_stride) return -ENOMEM;
+  const uint64_t whole = align_up(per_block, 256);
+  if (whole && a->blocks > SIZE_MAX / whole) return -ENOMEM;
+  *buf_stride = align_up(scan_window(per_block, a->threads), 256);
   CK(cudaSetDevice(ctx->cfg.device));
   const size_t need = (size_t)a->blocks * *buf_stride;
   if (need > ctx->scan_buf_bytes) {
@@ -1306,8 +1307,9 @@ int gfs_scan_path(gfs_ctx* ctx, const char* path, const gfs_scan_args* a, int64_
   CK(cudaSetDevice(ctx->cfg.device));
   const uint64_t per_block = std::min<uint64_t>(a->read_len, size);
   if (per_block > SIZE_MAX / 2) return -ENOMEM;
-  const uint64_t bs = align_up(per_block, 256);
-  if (bs && a->blocks > SIZE_MAX / bs) return -ENOMEM;
+  const uint64_t whole = align_up(per_block, 256);
+  if (whole && a->blocks > SIZE_MAX / whole) return -ENOMEM;
+  const uint64_t bs = align_up(scan_window(per_block, a->threads), 256);
   int rc = ensure_scan_buf(ctx, (size_t)a->blocks * bs);
   if (!rc) rc = ensure_paper_state(ctx, a->blocks);
   if (rc) return rc;

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(512, 1) k_scan_path(DevHandle g, const __grid_
   const int fid = dev::gopen(g, path.s, GFS_RDONLY);
   const long long size = fid >= 0 ? dev::gfstat_size(g, fid) : (long long)fid;
   for (unsigned long long s = b; s < nstrides; s += gridDim.x) {
-    dev::BufferSink<true> sink{buf, s * stride, {0ull, 0ull}};
+    dev::ScanSink<true> sink{buf, {0ull, 0ull}};
     const long long r = size < 0 ? size : dev::gread_impl(g, (int)b, fid, s * stride, read_len, sink);
     Sums acc = sink.acc;
     dev::block_sum2(acc.sum, acc.hash);
@@ -251,7 +251,9 @@ int scan_max_resident_blocks(uint32_t threads, bool fused, int device, int* out)
 namespace {
 
 constexpr size_t kStaticScratchBytes = 64ull << 20;  // GFS_STATIC_SCRATCH_BYTES in include/gfs.h
-static __device__ __align__(256) uint8_t g_scan_scratch[kStaticScratchBytes];
+// A read shorter than its block's window takes up to one word more than its length
+// rounded up to 256 bytes (scan_window), which is what the bound counts it with.
+static __device__ __align__(256) uint8_t g_scan_scratch[kStaticScratchBytes + kStaticScratchBytes / 16];
 
 // The context an address was looked up in: a caller that resets the device and
 // so creates a new primary context gets the array's address looked up again.
@@ -308,8 +310,9 @@ extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, in
   // and divide instead of multiplying, so that no size wraps around
   const uint64_t per_block = a->read_len < size ? a->read_len : size;
   if (per_block > kStaticScratchBytes) return -ENOSPC;
-  const uint64_t buf_stride = (per_block + 255) / 256 * 256;
-  if (buf_stride && a->blocks > kStaticScratchBytes / buf_stride) return -ENOSPC;  // beyond the static array
+  const uint64_t bound = (per_block + 255) / 256 * 256;
+  if (bound && a->blocks > kStaticScratchBytes / bound) return -ENOSPC;  // beyond the static array
+  const uint64_t buf_stride = gfs::scan_window(per_block, a->threads);
   if (nstrides == 0) return 0;
   if (!d_count || !d_sum || !d_hash) return -EINVAL;
   if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;

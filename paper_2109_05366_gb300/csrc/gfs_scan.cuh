@@ -86,14 +86,13 @@ __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsig
       }
       __syncthreads();
     }
-    dev::BufferSink<FUSED> sink{buf, off, {0ull, 0ull}};
+    dev::ScanSink<FUSED> sink{buf, {0ull, 0ull}};
     long long r = dev::gread_impl(g, (int)b, fid, off, read_len, sink);
     Sums acc = sink.acc;
     if (serialize) {  // wait until every request of this gread has been served
       block_quiesce(g);
       if (tid == 0) dev::st_rel64(&g.ctrl->ticket.v, s + 1);
     }
-    if (!FUSED && r > 0) checksum_range(buf, (unsigned long long)r, off, acc);
     dev::block_sum2(acc.sum, acc.hash);
     if (tid == 0) {
       cnt[s] = r;
