@@ -621,6 +621,7 @@ int gfs_shutdown(gfs_ctx* ctx) {
   if (!ctx) return 0;
   cudaSetDevice(ctx->cfg.device);
   if (ctx->server) gfs_serve_stop(ctx);
+  free_idle_server(ctx);
   if (ctx->io) {
     ctx->io->stop();
     delete ctx->io;

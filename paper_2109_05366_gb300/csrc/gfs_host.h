@@ -79,6 +79,7 @@ struct gfs_server;
 
 struct gfs_ctx {
   gfs_server* server = nullptr;  // running serving kernel, if any
+  gfs_server* idle_server = nullptr;  // the last one's memory, for the next start of at most its sizes
   gfs_config cfg{};
   gfs::DevHandle dev{};
   void* d_arena = nullptr;

@@ -64,7 +64,11 @@ struct Ctl {  // device memory
   Line active;
   Line adm_lock;
   Line last_work;
-  Line lost;  // completions dropped because the host left the completion ring full past the deadline
+};
+
+struct HostCtl {  // mapped pinned, after the rings
+  uint32_t stop, pad[15];
+  unsigned long long lost;  // completions dropped because the host left the completion ring full past the deadline
 };
 
 struct Handle {
@@ -72,7 +76,7 @@ struct Handle {
   ComplSlot* compl_;
   Req* req;
   Ctl* ctl;
-  const uint32_t* stop;  // mapped host flag
+  HostCtl* host;
   unsigned long long unit_bytes, idle_exit_ns;
   uint32_t sub_slots, compl_slots, max_req, units_cap, pages_per_unit, frame_budget;
 };
@@ -105,7 +109,7 @@ __device__ void complete(const DevHandle& g, const Handle& h, uint32_t r) {
     __nanosleep(256);
   }
   if (!claimed) {
-    atomicAdd(&h.ctl->lost.v, 1ull);
+    atomicAdd_system(&h.host->lost, 1ull);
     atomicAdd(&h.ctl->frames_reserved.v, (unsigned long long)(0ull - q.frames));
     atomicAdd(&h.ctl->active.v, ~0ull);
     dev::st_rel(&q.state, 0u);
@@ -218,7 +222,7 @@ __global__ void __launch_bounds__(512) k_serve(DevHandle g, Handle h) {
         s_len = end - s_off < h.unit_bytes ? end - s_off : h.unit_bytes;
         dev::st_rlx64(&h.ctl->last_work.v, dev::now_ns());
       } else {
-        const bool stopping = ld_sys32(h.stop) != 0;
+        const bool stopping = ld_sys32(&h.host->stop) != 0;
         const bool idle = dev::ld_rlx64(&h.ctl->active.v) == 0 &&
                           dev::ld_acq_sys64(&h.sub[dev::ld_rlx64(&h.ctl->sub_head.v) % h.sub_slots].seq) !=
                               dev::ld_rlx64(&h.ctl->sub_head.v) + 1;
@@ -271,12 +275,16 @@ __global__ void __launch_bounds__(512) k_serve(DevHandle g, Handle h) {
 using namespace gfs;
 using namespace gfs::serve;
 
+// Its memory outlives a serving kernel: gfs_serve_stop leaves it with the context
+// (one at most) and the next gfs_serve_start of no larger sizes takes it again.
 struct gfs_server {
   Handle h{};
   SubSlot* h_sub = nullptr;
   ComplSlot* h_compl = nullptr;
-  uint32_t* h_stop = nullptr;
+  HostCtl* h_ctl = nullptr;
   uint8_t* d_mem = nullptr;
+  uint8_t* h_mem = nullptr;  // mapped pinned: both rings and h_ctl
+  size_t d_bytes = 0, h_bytes = 0;
   cudaStream_t stream = nullptr;
   unsigned long long sub_tail = 0, compl_head = 0;
 };
@@ -287,9 +295,7 @@ int cerr(cudaError_t e) { return e == cudaSuccess ? 0 : (e == cudaErrorMemoryAll
 void free_server(gfs_server* s) {
   if (!s) return;
   if (s->d_mem) cudaFree(s->d_mem);
-  if (s->h_sub) cudaFreeHost(s->h_sub);
-  if (s->h_compl) cudaFreeHost(s->h_compl);
-  if (s->h_stop) cudaFreeHost(s->h_stop);
+  if (s->h_mem) cudaFreeHost(s->h_mem);
   delete s;
 }
 }  // namespace
@@ -310,9 +316,7 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   int rc = 0;
   rc = ensure_paper_state(ctx, sc->ctas);
   if (rc) return rc;
-  gfs_server* s = new (std::nothrow) gfs_server();
-  if (!s) return -ENOMEM;
-  Handle& h = s->h;
+  Handle h{};
   h.sub_slots = sc->queue_slots;
   h.compl_slots = sc->queue_slots;
   h.max_req = sc->max_requests;
@@ -326,34 +330,49 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   const size_t req_bytes = sizeof(Req) * h.max_req;
   const size_t ctl_off = (req_bytes + 255) / 256 * 256;
   const size_t total = ctl_off + sizeof(Ctl);
-  rc = cerr(cudaMalloc((void**)&s->d_mem, total));
-  if (!rc) rc = cerr(cudaMemset(s->d_mem, 0, total));
-  if (!rc) rc = cerr(cudaHostAlloc((void**)&s->h_sub, sizeof(SubSlot) * h.sub_slots, cudaHostAllocMapped));
-  if (!rc) rc = cerr(cudaHostAlloc((void**)&s->h_compl, sizeof(ComplSlot) * h.compl_slots, cudaHostAllocMapped));
-  if (!rc) rc = cerr(cudaHostAlloc((void**)&s->h_stop, 64, cudaHostAllocMapped));
+  // both rings and the host's control words in one mapped block
+  const size_t compl_off = (sizeof(SubSlot) * (size_t)h.sub_slots + 255) / 256 * 256;
+  const size_t hctl_off = compl_off + (sizeof(ComplSlot) * (size_t)h.compl_slots + 255) / 256 * 256;
+  const size_t host_total = hctl_off + sizeof(HostCtl);
+  gfs_server* s = ctx->idle_server;
+  ctx->idle_server = nullptr;
+  if (s && (s->d_bytes < total || s->h_bytes < host_total)) {
+    free_server(s);
+    s = nullptr;
+  }
+  if (!s) {
+    s = new (std::nothrow) gfs_server();
+    if (!s) return -ENOMEM;
+    rc = cerr(cudaMalloc((void**)&s->d_mem, total));
+    if (!rc) rc = cerr(cudaHostAlloc((void**)&s->h_mem, host_total, cudaHostAllocMapped));
+    if (rc) {
+      free_server(s);
+      return rc;
+    }
+    s->d_bytes = total;
+    s->h_bytes = host_total;
+  }
+  s->sub_tail = s->compl_head = 0;
+  s->stream = (cudaStream_t)stream;
+  void* p = nullptr;
+  rc = cerr(cudaHostGetDevicePointer(&p, s->h_mem, 0));
+  if (!rc) rc = cerr(cudaMemsetAsync(s->d_mem, 0, total, s->stream));
   if (rc) {
     free_server(s);
     return rc;
   }
-  memset(s->h_sub, 0, sizeof(SubSlot) * h.sub_slots);
-  memset(s->h_compl, 0, sizeof(ComplSlot) * h.compl_slots);
+  memset(s->h_mem, 0, host_total);
+  s->h_sub = (SubSlot*)s->h_mem;
+  s->h_compl = (ComplSlot*)(s->h_mem + compl_off);
+  s->h_ctl = (HostCtl*)(s->h_mem + hctl_off);
   for (uint32_t i = 0; i < h.sub_slots; ++i) s->h_sub[i].seq = i;
   for (uint32_t i = 0; i < h.compl_slots; ++i) s->h_compl[i].seq = i;
-  *s->h_stop = 0;
-  void* p = nullptr;
-  rc = cerr(cudaHostGetDevicePointer(&p, s->h_sub, 0));
   h.sub = (SubSlot*)p;
-  if (!rc) rc = cerr(cudaHostGetDevicePointer(&p, s->h_compl, 0));
-  h.compl_ = (ComplSlot*)p;
-  if (!rc) rc = cerr(cudaHostGetDevicePointer(&p, s->h_stop, 0));
-  h.stop = (const uint32_t*)p;
+  h.compl_ = (ComplSlot*)((uint8_t*)p + compl_off);
+  h.host = (HostCtl*)((uint8_t*)p + hctl_off);
   h.req = (Req*)s->d_mem;
   h.ctl = (Ctl*)(s->d_mem + ctl_off);
-  if (rc) {
-    free_server(s);
-    return rc;
-  }
-  s->stream = (cudaStream_t)stream;
+  s->h = h;
   DevHandle g = ctx->dev;
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames : (uint32_t)(in_use + 1);
   k_serve<<<sc->ctas, sc->threads, 0, s->stream>>>(g, h);
@@ -412,9 +431,10 @@ extern "C" int gfs_serve_stop(gfs_ctx* ctx) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   gfs_server* s = ctx->server;
   if (!s) return 0;
-  __atomic_store_n(s->h_stop, 1u, __ATOMIC_RELEASE);
+  __atomic_store_n(&s->h_ctl->stop, 1u, __ATOMIC_RELEASE);
   // completions not polled by now are discarded: keep the ring drained so no CTA
   // waits for a slot while the kernel finishes its last requests
+  const auto t0 = std::chrono::steady_clock::now();
   cudaError_t q;
   while ((q = cudaStreamQuery(s->stream)) == cudaErrorNotReady) {
     for (;;) {
@@ -424,12 +444,18 @@ extern "C" int gfs_serve_stop(gfs_ctx* ctx) {
       __atomic_store_n(&cs->seq, c + s->h.compl_slots, __ATOMIC_RELEASE);
       s->compl_head = c + 1;
     }
-    usleep(100);
+    // an idle kernel ends within tens of microseconds
+    if (std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(1)) usleep(100);
   }
-  int rc = cerr(q);
-  unsigned long long lost = 0;
-  if (!rc) rc = cerr(cudaMemcpy(&lost, &s->h.ctl->lost.v, 8, cudaMemcpyDeviceToHost));
-  free_server(s);
+  const int rc = cerr(q);
+  const unsigned long long lost = __atomic_load_n(&s->h_ctl->lost, __ATOMIC_ACQUIRE);
   ctx->server = nullptr;
+  if (rc) free_server(s);
+  else ctx->idle_server = s;
   return rc ? rc : (lost ? -ENOBUFS : 0);
+}
+
+void free_idle_server(gfs_ctx* ctx) {
+  free_server(ctx->idle_server);
+  ctx->idle_server = nullptr;
 }
