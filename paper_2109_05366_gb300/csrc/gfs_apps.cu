@@ -29,6 +29,7 @@ constexpr uint32_t kSmemBins = 8192;  // histogram bins kept in shared memory (t
 // three times (out of the cache, into the buffer, back in): a cached 16384 x 8192 matrix
 // took 303 us that way and takes 135 us in place.
 struct RowdotSink {
+  static constexpr bool kArrive = true;
   const float4* vec;
   float* out;  // the gread's first row
   float4* carry;  // shared memory, 2 x 32; one half is read while the other is written
@@ -149,7 +150,7 @@ struct RowdotSink {
 
 // Block b reads stripes b, b + B, ...; a stripe is `stripe_rows` rows and is read
 // in pieces of `read_len` bytes (whole rows).
-__global__ void __launch_bounds__(kThreads) k_rowdot(DevHandle g, int fid, uint32_t rows, uint32_t cols,
+__global__ void __launch_bounds__(kThreads, 2) k_rowdot(DevHandle g, int fid, uint32_t rows, uint32_t cols,
                                                      const float* __restrict__ vec, float* __restrict__ out,
                                                      uint32_t stripe_rows, unsigned long long read_len,
                                                      unsigned long long* stripe_sum,
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(kThreads) k_rowdot(DevHandle g, int fid, uint3
 // buffer and the match, 1602 us without; 1280 us is the host link.)  A last value of fewer
 // than four bytes is not counted.
 struct HistSink {
+  static constexpr bool kArrive = true;
   uint32_t* sh;
   uint32_t* hist;
   uint32_t nbins;
@@ -235,7 +237,7 @@ struct HistSink {
 };
 
 // Block b reads pieces b, b + B, ... of the int32 file and counts values.
-__global__ void __launch_bounds__(kThreads) k_histogram(DevHandle g, int fid, unsigned long long size, uint32_t nbins,
+__global__ void __launch_bounds__(kThreads, 2) k_histogram(DevHandle g, int fid, unsigned long long size, uint32_t nbins,
                                                         uint32_t* __restrict__ hist, unsigned long long read_len,
                                                         unsigned long long* sums, long long* status) {
   __shared__ uint32_t sh[kSmemBins];
