@@ -283,6 +283,7 @@ extern "C" int gfs_rowdot(gfs_ctx* ctx, int fid, uint32_t rows, uint32_t cols, c
   if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;
   const int rc = ensure_paper_state(ctx, blocks);
   if (rc) return rc;
+  note_read(ctx, fid);
   DevHandle g = ctx->dev;
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
                                       : blocks * (uint32_t)((read_len + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;
@@ -301,6 +302,7 @@ extern "C" int gfs_histogram(gfs_ctx* ctx, int fid, uint32_t nbins, uint32_t* d_
   if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;
   const int rc = ensure_paper_state(ctx, blocks);
   if (rc) return rc;
+  note_read(ctx, fid);
   DevHandle g = ctx->dev;
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
                                       : blocks * (uint32_t)((read_len + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;

@@ -1082,6 +1082,7 @@ int gfs_reset_cache(gfs_ctx* ctx, void* stream) {
   int rc = launch_reset(ctx->dev, s);
   if (rc) return rc;
   CK(cudaStreamSynchronize(s));
+  for (auto& f : ctx->files) __atomic_store_n(&f.maybe_cached, (uint8_t)0, __ATOMIC_RELAXED);
   return reclaim_retired(ctx, true);  // ids closed on the device: their pages are gone now
 }
 
@@ -1242,6 +1243,7 @@ static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t*
   if (a->threads != 128 && a->threads != 256 && a->threads != 512) return -EINVAL;
   const uint64_t size = ctx->files[fid].size;
   *nstrides = size ? (size + a->stride - 1) / a->stride : 0;
+  note_read(ctx, fid);
   // a gread never delivers more than the file holds; the checks divide so that
   // no size wraps around
   const uint64_t per_block = std::min<uint64_t>(a->read_len, size);
@@ -1328,6 +1330,7 @@ int gfs_scan_path(gfs_ctx* ctx, const char* path, const gfs_scan_args* a, int64_
 int gfs_device_handle(gfs_ctx* ctx, uint32_t blocks, uint64_t read_len, void* out, uint64_t cap) {
   if (!ctx || !out || blocks == 0 || read_len == 0) return -EINVAL;
   if (cap < sizeof(DevHandle)) return -ENOSPC;
+  __atomic_store_n(&ctx->handle_out, (uint8_t)1, __ATOMIC_RELAXED);
   DevHandle g = ctx->dev;
   const uint64_t pages_per_read = (read_len >> ctx->dev.page_shift) + ((read_len & (ctx->cfg.page_size - 1)) != 0);
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
@@ -1438,7 +1441,8 @@ int gfs_read_many(gfs_ctx* ctx, int fid, uint32_t n, const uint64_t* d_off, cons
   if (prc) return prc;
   DevHandle g = ctx->dev;
   g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames : blocks + 1;
-  return launch_read_many(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, (cudaStream_t)stream);
+  return launch_read_many(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, note_read(ctx, fid),
+                          (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------- CPU-I/O baseline

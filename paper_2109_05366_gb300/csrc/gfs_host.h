@@ -41,6 +41,9 @@ struct HostFile {
   // closed on the device: the id keeps its cached pages (and its descriptor)
   // until they are dropped at a quiet point
   bool retired = false;
+  // a kernel that may bring pages of the file into the cache was launched since they
+  // were last dropped (relaxed atomic access; only picks a kernel instance)
+  uint8_t maybe_cached = 0;
 };
 
 class IoService;
@@ -60,7 +63,7 @@ int launch_scan_path(const DevHandle& g, const PathArg& path, const gfs_scan_arg
 int launch_purge(const DevHandle& g, uint32_t fid, cudaStream_t s);
 int launch_read_many(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                      const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
-                     cudaStream_t s);
+                     bool cold, cudaStream_t s);
 int launch_checksum(const uint8_t* d_file, uint64_t size, uint64_t stride, uint64_t read_len, int64_t* d_count,
                     uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
 int scan_max_resident_blocks(uint32_t threads, bool fused, int device, int* out);
@@ -78,6 +81,7 @@ namespace gfs {
 struct gfs_server;
 
 struct gfs_ctx {
+  uint8_t handle_out = 0;        // user kernels may read files (gfs_device_handle): as maybe_cached, for all
   gfs_server* server = nullptr;  // running serving kernel, if any
   gfs_server* idle_server = nullptr;  // the last one's memory, for the next start of at most its sizes
   gfs_config cfg{};
@@ -111,3 +115,11 @@ struct gfs_ctx {
   std::mutex files_mu;             // HostFile fields read by the host I/O threads
   std::mutex dev_open_mu;          // device opens and closes, one at a time
 };
+
+// Call when launching a kernel that reads fid.  Returns whether none of the file's pages
+// can be cached yet (no such launch since they were last dropped).
+inline bool note_read(gfs_ctx* ctx, int fid) {
+  gfs::HostFile& f = ctx->files[fid];
+  return !__atomic_exchange_n(&f.maybe_cached, (uint8_t)1, __ATOMIC_RELAXED) && !f.by_device &&
+         !__atomic_load_n(&ctx->handle_out, __ATOMIC_RELAXED);
+}

@@ -163,7 +163,8 @@ GFS_HD inline uint32_t slot_stride(uint32_t max_pages) {
 constexpr uint32_t SCAN_UNITS = 4, SCAN_UNIT_BYTES = 4096;
 inline uint64_t scan_window(uint64_t read_bytes, uint32_t threads) {
   const uint64_t window = (uint64_t)(threads / 32) * SCAN_UNITS * SCAN_UNIT_BYTES;
-  return read_bytes >= window ? window : (read_bytes + 30) / 16 * 16 < window ? (read_bytes + 30) / 16 * 16 : window;
+  const uint64_t whole = (read_bytes + 15 + 15) / 16 * 16;
+  return whole < window ? whole : window;
 }
 
 // Handle passed by value to every kernel.  Plain data only.

@@ -199,13 +199,13 @@ int launch_purge(const DevHandle& g, uint32_t fid, cudaStream_t s) {
 
 int launch_read_many(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                      const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
-                     cudaStream_t s) {
+                     bool cold, cudaStream_t s) {
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return -19;
   if (scan_variant(threads, blocks, device) == 0)
     launch_read_many_wide(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, s);
   else
-    launch_read_many_narrow(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, s);
+    launch_read_many_narrow(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, cold, s);
   return cuda_err(cudaGetLastError());
 }
 
@@ -319,6 +319,7 @@ extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, in
   if ((ctx->cfg.mode == GFS_MODE_PAPER || ctx->cfg.replacement == GFS_REPL_TB_LRA) &&
       ctx->dev.paper_streams < a->blocks)
     return -ENOTSUP;  // the per-block state would have to be allocated
+  note_read(ctx, fid);
   void* scratch = nullptr;
   int rc = static_scratch(ctx->cfg.device, &scratch);
   if (rc) return rc;

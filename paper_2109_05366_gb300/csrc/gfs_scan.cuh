@@ -104,17 +104,21 @@ __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsig
   block_help_drain(g);
 }
 
-// Independent greads (Section 2.2): block b serves reads b, b + B, ...; read i
-// copies len[i] bytes at off[i] to buf + dst[i] and stores the return value in
-// ret[i].  MAXT, MINB as for k_scan: a small read costs a block mostly control-path
+// Independent greads (Section 2.2): block b serves reads b, b + B, ... of the
+// list.  MAXT, MINB as for k_scan: a small read costs a block mostly control-path
 // latency, so the reads in flight grow with the blocks resident per SM.
-template <int MAXT, int MINB>
-__global__ void __launch_bounds__(MAXT, MINB) k_read_many(DevHandle g, int fid, uint32_t n, const uint64_t* off,
-                                                    const uint64_t* len, const uint64_t* dst, uint8_t* buf,
-                                                    long long* ret) {
-  for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
-    long long r = dev::gread(g, (int)blockIdx.x, fid, off[i], len[i], buf + dst[i]);
-    if (threadIdx.x == 0) ret[i] = r;
+// BATCH: reads of cached pages go in batches.  The <256, 4> instance also exists without,
+// for lists on files of which nothing can be cached yet: there the batches' call makes the
+// register allocator spill what gread holds (131072 random 4 KiB pages from the host:
+// 2337 us with, 2223 us without).
+template <bool BATCH, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_read_many(DevHandle g, int fid, dev::ReadList list) {
+  dev::ReadCursor at{blockIdx.x, 0u, 1u};
+  for (unsigned long long i = blockIdx.x;; i += gridDim.x) {
+    if (BATCH) i = dev::read_batches(g, list, fid, at);
+    if (i >= list.n) break;
+    long long r = dev::gread(g, (int)blockIdx.x, fid, list.off[i], list.len[i], list.buf + list.dst[i]);
+    if (threadIdx.x == 0) list.ret[i] = r;
     __syncthreads();
   }
   block_help_drain(g);
@@ -143,6 +147,6 @@ void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64
                            cudaStream_t s);
 void launch_read_many_narrow(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                              const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
-                             cudaStream_t s);
+                             bool cold, cudaStream_t s);
 
 }  // namespace gfs

@@ -17,8 +17,10 @@ cudaError_t scan_occupancy_narrow(bool fused, int threads, int* per_sm) {
 
 void launch_read_many_narrow(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                       const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
-                      cudaStream_t s) {
-  k_read_many<256, 4><<<blocks, threads, 0, s>>>(g, fid, n, d_off, d_len, d_dst, d_buf, (long long*)d_ret);
+                      bool cold, cudaStream_t s) {
+  const dev::ReadList list{d_off, d_len, d_dst, d_buf, (long long*)d_ret, n};
+  if (cold) k_read_many<false, 256, 4><<<blocks, threads, 0, s>>>(g, fid, list);
+  else k_read_many<true, 256, 4><<<blocks, threads, 0, s>>>(g, fid, list);
 }
 
 }  // namespace gfs

@@ -392,6 +392,7 @@ extern "C" int gfs_submit_scan(gfs_ctx* ctx, int fid, uint64_t off, uint64_t len
   const unsigned long long t = s->sub_tail;
   SubSlot* ss = &s->h_sub[t % s->h.sub_slots];
   if (__atomic_load_n(&ss->seq, __ATOMIC_ACQUIRE) != t) return -EAGAIN;  // ring full
+  note_read(ctx, fid);
   ss->fid = (uint32_t)fid;
   ss->off = off;
   ss->len = len;
