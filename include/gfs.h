@@ -216,7 +216,7 @@ typedef struct gfs_scan_args {
   uint32_t blocks;    /* threadblocks (gread streams) */
   uint32_t threads;   /* threads per block: 128, 256 or 512 */
   uint32_t serialize; /* 1: one gread at a time in stride order, each waiting for its requests (exact policy traces) */
-  uint32_t fused;     /* 1: checksum while copying out of the cache (no user-buffer re-read) */
+  uint32_t fused;     /* 0 or 1: both deliver into the block's window in shared memory and sum it there */
   uint32_t reserved[4];
 } gfs_scan_args;
 
@@ -326,22 +326,12 @@ int gfs_scan_host(gfs_ctx* ctx, int fid, const gfs_scan_args* args, int64_t* h_c
  * service of this library.  Some callers cannot call cudaMalloc while they
  * run: serving loops that must not stall other streams (cudaMalloc and cudaFree
  * can synchronise the device), and code that owns all of a device's memory
- * through its own allocator and budget.  gfs_scan may allocate its
- * per-threadblock gread buffers on first use or growth; this call never
- * allocates (no cudaMalloc, cudaFree or allocating library routine): the
- * buffers live in a file-scope device array of GFS_STATIC_SCRATCH_BYTES that
- * every device loading the library holds until the process exits.
+ * through its own allocator and budget.  This call never allocates (no
+ * cudaMalloc, cudaFree or allocating library routine): the blocks keep what they
+ * read in shared memory.
  *   - blocks * round_up(min(read_len, file size), 256) must fit in
  *     GFS_STATIC_SCRATCH_BYTES, else the call returns -ENOSPC and launches
  *     nothing.
- *   - The first call on a device looks the array's device address up (with that
- *     device made current) and caches it per device and CUDA context; make that
- *     first call before any stream capture.  A caller that resets the device
- *     (cudaDeviceReset) loses every context of this library anyway; the address
- *     is then looked up again in the new context.
- *   - Every call shares the one array and leaves its contents behind; nothing
- *     in it needs to start at zero.  Calls whose kernels overlap on the GPU
- *     race on the array: serialise them (one stream, or events).
  *   - With GFS_MODE_PAPER or GFS_REPL_TB_LRA the context keeps per-threadblock
  *     state that an allocating call sizes: -ENOTSUP until a gfs_scan (or
  *     gfs_scan_path, gfs_read_many) with at least `blocks` threadblocks has run

@@ -2349,51 +2349,72 @@ struct SumSink {
   }
 };
 
-// The stride scan's consumer: a gread delivered through a window of the block's
-// buffer, kScanUnits units for each warp, that is read back as it fills (FUSED:
-// checksummed on the way in instead, without the read back).
-// Bound by HBM: the window stays in L2 (296 blocks of 256 threads: 37 MiB), so a cached
-// byte moves over HBM once.  Buffers of a whole read (310 MB) did not: each byte was
-// read, written, evicted and read again.  A cached 1 GiB scan, 296 blocks, 512 KiB pages:
-// 579 us with whole buffers, 296 us with windows.
-// A warp reads back only what it delivered, so the block does not wait for itself;
-// unit u always goes to the same cell, by the same warp.
-constexpr uint32_t kScanUnits = SCAN_UNITS;
-static_assert(SCAN_UNIT_BYTES == 1u << kUnitShift, "a cell holds a unit");
-template <bool FUSED>
-struct ScanSink {
+// The consumer of a block that wants the checksums: a gread delivered into a window in
+// shared memory, STAGES units for each warp, and summed from there.  Each lane copies its
+// own words of a unit asynchronously (cp.async, past L1 and the registers) and reads only
+// those back, so a warp needs no barrier: it sums a unit while its next STAGES - 1 are on
+// their way, and then has that cell filled again.
+// Bound by HBM reads.  A window in device memory that stayed in L2 was bound by L2, which
+// moved each byte three times (out of the cache, into the window, back): a cached 1 GiB
+// scan by 296 blocks, 512 KiB pages, took 296 us that way (579 us with buffers of a whole
+// read), also with the next unit's loads under way, and takes 184 us from here.
+__device__ __forceinline__ uint8_t* window_memory() {
+  extern __shared__ uint4 s_window[];
+  return reinterpret_cast<uint8_t*>(s_window);
+}
+__device__ __forceinline__ void async_word(uint32_t to, const uint8_t* from) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(from) : "memory");
+}
+template <int STAGES>
+struct WindowSink {
   static constexpr bool kArrive = true;
-  uint8_t* buf;  // scan_window() bytes, 16-byte aligned
   Sums acc;
+
+  // Start copying the unit at file offset `at` into the lane's words of a cell.
+  __device__ __forceinline__ void fetch(const DevHandle& g, const RunView& r, unsigned long long at,
+                                        uint32_t cell) const {
+    const unsigned long long rel = at - (r.p << g.page_shift);
+    const uint32_t lane = threadIdx.x & 31u;
+    if (((uint32_t)rel & (g.page_size - 1u)) + (1u << kUnitShift) <= g.page_size && at + (1u << kUnitShift) <= r.hi) {
+      const uint8_t* p = run_at(g, r, rel) + 16 * lane;  // whole, in one page
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) async_word(cell + 512 * k, p + 512 * k);
+    } else {
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k)
+        if (at + 16 * lane + 512 * k < r.hi) async_word(cell + 512 * k, run_at(g, r, rel + 16 * lane + 512 * k));
+    }
+  }
+
   __device__ __noinline__ void take(const DevHandle& g, const RunView& r) {
     const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31u, units = run_units(r);
-    const unsigned long long o = r.lo & ~15ull;
+    const unsigned long long step = (unsigned long long)nw << kUnitShift;
+    unsigned long long at = (r.lo & ~15ull) + ((unsigned long long)w << kUnitShift);
+    uint8_t* mine = window_memory() + ((size_t)w * STAGES << kUnitShift) + 16 * lane;
+    const uint32_t cells = (uint32_t)__cvta_generic_to_shared(mine);
     Sums part{0ull, 0ull};
-    for (uint32_t u0 = w; u0 < units; u0 += kScanUnits * nw) {
-#pragma unroll 1
-      for (uint32_t i = 0; i < kScanUnits && u0 + i * nw < units; ++i) {
-        const unsigned long long at = o + ((unsigned long long)(u0 + i * nw) << kUnitShift);
-        uint4* cell = reinterpret_cast<uint4*>(buf + ((size_t)(w + i * nw) << kUnitShift)) + lane;
-        uint4 v[8];
-        load_unit(g, r, at, v);
 #pragma unroll
-        for (uint32_t k = 0; k < 8; ++k)
-          if (at + 16 * lane + 512 * k < r.hi) cell[32 * k] = v[k];
-        if (FUSED) unit_sums(part, v, at);
-      }
-      if (FUSED) continue;
-      __syncwarp();
-#pragma unroll 1
-      for (uint32_t i = 0; i < kScanUnits && u0 + i * nw < units; ++i) {
-        const unsigned long long at = o + ((unsigned long long)(u0 + i * nw) << kUnitShift);
-        const uint4* cell = reinterpret_cast<const uint4*>(buf + ((size_t)(w + i * nw) << kUnitShift)) + lane;
-        uint4 v[8];
-#pragma unroll
-        for (uint32_t k = 0; k < 8; ++k)
-          v[k] = at + 16 * lane + 512 * k < r.hi ? cell[32 * k] : make_uint4(0u, 0u, 0u, 0u);
-        unit_sums(part, v, at);
-      }
+    for (int i = 0; i < STAGES; ++i) {
+      if (w + i * nw < units) fetch(g, r, at + i * step, cells + (i << kUnitShift));
+      asm volatile("cp.async.commit_group;" ::: "memory");
     }
+    uint32_t c = 0;  // the cell of unit u
+    for (uint32_t u = w; u < units; u += nw, at += step) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 1) : "memory");
+      const uint4* x = reinterpret_cast<const uint4*>(mine + ((size_t)c << kUnitShift));
+      uint4 v[8];
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) v[k] = x[32 * k];
+      if (at < r.lo || at + (1u << kUnitShift) > r.hi) {  // bytes outside the view, and words not copied
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) v[k] = clip_word(v[k], at + 16 * lane + 512 * k, r.lo, r.hi);
+      }
+      unit_sums(part, v, at);
+      if (u + STAGES * nw < units) fetch(g, r, at + STAGES * step, cells + (c << kUnitShift));
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      c = c + 1 < STAGES ? c + 1 : 0;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     acc.sum += part.sum;
     acc.hash += part.hash;
   }

@@ -635,7 +635,6 @@ int gfs_shutdown(gfs_ctx* ctx) {
   if (ctx->h_cancel) cudaFreeHost(ctx->h_cancel);
   if (ctx->d_arena) cudaFree(ctx->d_arena);
   if (ctx->d_frames) cudaFree(ctx->d_frames);
-  if (ctx->d_scan_buf) cudaFree(ctx->d_scan_buf);
   if (ctx->d_paper) cudaFree(ctx->d_paper);
   if (ctx->d_out) cudaFree(ctx->d_out);
   if (ctx->h_out) cudaFreeHost(ctx->h_out);
@@ -1222,21 +1221,9 @@ int ensure_paper_state(gfs_ctx* ctx, uint32_t streams) {
   return 0;
 }
 
-int ensure_scan_buf(gfs_ctx* ctx, size_t need) {
-  if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;
-  if (need <= ctx->scan_buf_bytes) return 0;
-  if (ctx->d_scan_buf) cudaFree(ctx->d_scan_buf);
-  ctx->d_scan_buf = nullptr;
-  ctx->scan_buf_bytes = 0;
-  CK(cudaMalloc((void**)&ctx->d_scan_buf, need));
-  ctx->scan_buf_bytes = need;
-  return 0;
-}
-
 extern "C" {
 
-static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t* nstrides, uint64_t* buf_stride,
-                        DevHandle* g) {
+static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t* nstrides, DevHandle* g) {
   if (!ctx || !a) return -EINVAL;
   if (fid < 0 || (size_t)fid >= ctx->files.size() || !ctx->files[fid].open) return -EBADF;
   if (a->stride == 0 || a->read_len == 0 || a->blocks == 0) return -EINVAL;
@@ -1250,16 +1237,7 @@ static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t*
   if (per_block > SIZE_MAX / 2) return -ENOMEM;
   const uint64_t whole = align_up(per_block, 256);
   if (whole && a->blocks > SIZE_MAX / whole) return -ENOMEM;
-  *buf_stride = align_up(scan_window(per_block, a->threads), 256);
   CK(cudaSetDevice(ctx->cfg.device));
-  const size_t need = (size_t)a->blocks * *buf_stride;
-  if (need > ctx->scan_buf_bytes) {
-    if (ctx->d_scan_buf) cudaFree(ctx->d_scan_buf);
-    ctx->d_scan_buf = nullptr;
-    ctx->scan_buf_bytes = 0;
-    CK(cudaMalloc((void**)&ctx->d_scan_buf, need));
-    ctx->scan_buf_bytes = need;
-  }
   {
     int prc = ensure_paper_state(ctx, a->blocks);
     if (prc) return prc;
@@ -1272,7 +1250,7 @@ static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t*
                                                                       : a->blocks * pages_per_read + 1);
   if (a->serialize) {
     int maxb = 0;
-    int rc = scan_max_resident_blocks(a->threads, a->fused != 0, ctx->cfg.device, &maxb);
+    int rc = scan_max_resident_blocks(a->threads, ctx->cfg.device, &maxb);
     if (rc) return rc;
     if ((int)a->blocks > maxb) return -EINVAL;  // every block must be resident to take its turn
   }
@@ -1281,15 +1259,15 @@ static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t*
 
 int gfs_scan(gfs_ctx* ctx, int fid, const gfs_scan_args* a, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash,
              void* stream) {
-  uint64_t ns = 0, bs = 0;
+  uint64_t ns = 0;
   DevHandle g;
-  int rc = scan_prepare(ctx, fid, a, &ns, &bs, &g);
+  int rc = scan_prepare(ctx, fid, a, &ns, &g);
   if (rc) return rc;
   if (ns == 0) return 0;
   if (!d_count || !d_sum || !d_hash) return -EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   if (a->serialize) CK(cudaMemsetAsync(&g.ctrl->ticket.v, 0, 8, s));
-  return launch_scan(g, fid, *a, ns, ctx->d_scan_buf, bs, d_count, d_sum, d_hash, s);
+  return launch_scan(g, fid, *a, ns, d_count, d_sum, d_hash, s);
 }
 
 int gfs_scan_path(gfs_ctx* ctx, const char* path, const gfs_scan_args* a, int64_t* d_count, uint64_t* d_sum,
@@ -1312,9 +1290,7 @@ int gfs_scan_path(gfs_ctx* ctx, const char* path, const gfs_scan_args* a, int64_
   if (per_block > SIZE_MAX / 2) return -ENOMEM;
   const uint64_t whole = align_up(per_block, 256);
   if (whole && a->blocks > SIZE_MAX / whole) return -ENOMEM;
-  const uint64_t bs = align_up(scan_window(per_block, a->threads), 256);
-  int rc = ensure_scan_buf(ctx, (size_t)a->blocks * bs);
-  if (!rc) rc = ensure_paper_state(ctx, a->blocks);
+  const int rc = ensure_paper_state(ctx, a->blocks);
   if (rc) return rc;
   DevHandle g = ctx->dev;
   const uint64_t pages_per_read = (a->read_len >> ctx->dev.page_shift) + ((a->read_len & (ctx->cfg.page_size - 1)) != 0);
@@ -1324,7 +1300,7 @@ int gfs_scan_path(gfs_ctx* ctx, const char* path, const gfs_scan_args* a, int64_
   PathArg pa;
   memset(pa.s, 0, sizeof(pa.s));
   memcpy(pa.s, path, len);
-  return launch_scan_path(g, pa, *a, ns, ctx->d_scan_buf, bs, d_count, d_sum, d_hash, (cudaStream_t)stream);
+  return launch_scan_path(g, pa, *a, ns, d_count, d_sum, d_hash, (cudaStream_t)stream);
 }
 
 int gfs_device_handle(gfs_ctx* ctx, uint32_t blocks, uint64_t read_len, void* out, uint64_t cap) {
@@ -1342,9 +1318,9 @@ int gfs_device_handle(gfs_ctx* ctx, uint32_t blocks, uint64_t read_len, void* ou
 
 int gfs_scan_host(gfs_ctx* ctx, int fid, const gfs_scan_args* a, int64_t* h_count, uint64_t* h_sum, uint64_t* h_hash,
                   void* stream) {
-  uint64_t ns = 0, bs = 0;
+  uint64_t ns = 0;
   DevHandle g;
-  int rc = scan_prepare(ctx, fid, a, &ns, &bs, &g);
+  int rc = scan_prepare(ctx, fid, a, &ns, &g);
   if (rc) return rc;
   if (ns == 0) return 0;
   if (!h_count || !h_sum || !h_hash) return -EINVAL;
@@ -1367,7 +1343,7 @@ int gfs_scan_host(gfs_ctx* ctx, int fid, const gfs_scan_args* a, int64_t* h_coun
   uint64_t* dsum = (uint64_t*)(ctx->d_out + ns * 8);
   uint64_t* dh = (uint64_t*)(ctx->d_out + ns * 16);
   if (a->serialize) CK(cudaMemsetAsync(&g.ctrl->ticket.v, 0, 8, s));
-  rc = launch_scan(g, fid, *a, ns, ctx->d_scan_buf, bs, dc, dsum, dh, s);
+  rc = launch_scan(g, fid, *a, ns, dc, dsum, dh, s);
   if (!rc) rc = cuda_err(cudaMemcpyAsync(ctx->h_out, ctx->d_out, need, cudaMemcpyDeviceToHost, s));
   int rc2 = cuda_err(cudaStreamSynchronize(s));
   if (!rc && !rc2) {
@@ -1380,11 +1356,11 @@ int gfs_scan_host(gfs_ctx* ctx, int fid, const gfs_scan_args* a, int64_t* h_coun
 
 int gfs_scan_graph(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint32_t reps, int64_t* d_count, uint64_t* d_sum,
                    uint64_t* d_hash, void* stream) {
-  uint64_t ns = 0, bs = 0;
+  uint64_t ns = 0;
   DevHandle g;
   if (ctx && ctx->cfg.xfer == GFS_XFER_DMA) return -ENOTSUP;
   if (reps == 0) return -EINVAL;
-  int rc = scan_prepare(ctx, fid, a, &ns, &bs, &g);  // allocates the scan buffers before capture
+  int rc = scan_prepare(ctx, fid, a, &ns, &g);  // allocates what it needs before capture
   if (rc) return rc;
   if (ns == 0) return 0;
   if (!d_count || !d_sum || !d_hash) return -EINVAL;
@@ -1413,7 +1389,7 @@ int gfs_scan_graph(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint32_t reps,
       }
       if (!rc) rc = launch_reset(ctx->dev, cs);
       if (!rc && a->serialize) rc = cuda_err(cudaMemsetAsync(&g.ctrl->ticket.v, 0, 8, cs));
-      if (!rc) rc = launch_scan(g, fid, *a, ns, ctx->d_scan_buf, bs, d_count, d_sum, d_hash, cs);
+      if (!rc) rc = launch_scan(g, fid, *a, ns, d_count, d_sum, d_hash, cs);
     }
     const int rc2 = cuda_err(cudaStreamEndCapture(cs, &graph));
     if (!rc) rc = rc2;

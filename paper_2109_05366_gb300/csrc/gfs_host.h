@@ -51,27 +51,24 @@ class IoService;
 // Entry points of the device code, implemented in gfs_kernels.cu.
 int launch_reset(const DevHandle& g, cudaStream_t s);
 int launch_drain(const DevHandle& g, cudaStream_t s);
-int launch_scan(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides, uint8_t* bufs,
-                uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
+int launch_scan(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
+                int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
 // A path passed by value as a kernel parameter (readable through a pointer).
 struct PathArg {
   char s[GFS_PATH_MAX];
 };
 int launch_scan_path(const DevHandle& g, const PathArg& path, const gfs_scan_args& a, unsigned long long nstrides,
-                     uint8_t* bufs, uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash,
-                     cudaStream_t s);
+                     int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
 int launch_purge(const DevHandle& g, uint32_t fid, cudaStream_t s);
 int launch_read_many(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                      const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
                      bool cold, cudaStream_t s);
 int launch_checksum(const uint8_t* d_file, uint64_t size, uint64_t stride, uint64_t read_len, int64_t* d_count,
                     uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
-int scan_max_resident_blocks(uint32_t threads, bool fused, int device, int* out);
+int scan_max_resident_blocks(uint32_t threads, int device, int* out);
 int launch_pull_probe(const uint8_t* src, uint8_t* dst, uint64_t n, cudaStream_t s);
 }  // namespace gfs
 struct gfs_ctx;
-// Grow the context's per-block gread buffers to at least `bytes` (before a launch).
-int ensure_scan_buf(gfs_ctx* ctx, size_t bytes);
 // GFS_MODE_PAPER: private buffers and LRA queues for `streams` streams (before a launch).
 int ensure_paper_state(gfs_ctx* ctx, uint32_t streams);
 namespace gfs {
@@ -97,8 +94,6 @@ struct gfs_ctx {
   uint32_t* h_bcount = nullptr;
   std::vector<gfs::HostFile> files;
   gfs::IoService* io = nullptr;
-  uint8_t* d_scan_buf = nullptr;  // per-block gread buffers of gfs_scan
-  size_t scan_buf_bytes = 0;
   cudaGraphExec_t graph = nullptr;  // gfs_scan_graph: cached executable and its key
   unsigned long long graph_key[8] = {};
   uint8_t* d_paper = nullptr;       // GFS_MODE_PAPER state (private buffers, metadata, LRA queues)

@@ -158,15 +158,6 @@ GFS_HD inline uint32_t slot_stride(uint32_t max_pages) {
   return (b + 63) & ~63u;
 }
 
-// Bytes of buffer a block of the stride scan needs: its window (16 KiB for each
-// warp), or the whole read with the words its ends fall in where that is less.
-constexpr uint32_t SCAN_UNITS = 4, SCAN_UNIT_BYTES = 4096;
-inline uint64_t scan_window(uint64_t read_bytes, uint32_t threads) {
-  const uint64_t window = (uint64_t)(threads / 32) * SCAN_UNITS * SCAN_UNIT_BYTES;
-  const uint64_t whole = (read_bytes + 15 + 15) / 16 * 16;
-  return whole < window ? whole : window;
-}
-
 // Handle passed by value to every kernel.  Plain data only.
 struct DevHandle {
   // configuration

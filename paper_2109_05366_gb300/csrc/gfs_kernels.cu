@@ -19,14 +19,13 @@ namespace gfs {
 __global__ void __launch_bounds__(512, 1) k_scan_path(DevHandle g, const __grid_constant__ PathArg path,
                                                     unsigned long long stride,
                                                     unsigned long long read_len, unsigned long long nstrides,
-                                                    uint8_t* bufs, unsigned long long buf_stride, long long* cnt,
-                                                    unsigned long long* sum, unsigned long long* hash) {
+                                                    long long* cnt, unsigned long long* sum,
+                                                    unsigned long long* hash) {
   const uint32_t b = blockIdx.x, tid = threadIdx.x;
-  uint8_t* buf = bufs + (size_t)b * buf_stride;
   const int fid = dev::gopen(g, path.s, GFS_RDONLY);
   const long long size = fid >= 0 ? dev::gfstat_size(g, fid) : (long long)fid;
   for (unsigned long long s = b; s < nstrides; s += gridDim.x) {
-    dev::ScanSink<true> sink{buf, {0ull, 0ull}};
+    dev::WindowSink<scan_stages(1)> sink{{0ull, 0ull}};
     const long long r = size < 0 ? size : dev::gread_impl(g, (int)b, fid, s * stride, read_len, sink);
     Sums acc = sink.acc;
     dev::block_sum2(acc.sum, acc.hash);
@@ -172,23 +171,23 @@ static int scan_variant(uint32_t threads, uint32_t blocks, int device) {
   return blocks <= 2u * (uint32_t)n ? 0 : 1;
 }
 
-int launch_scan(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides, uint8_t* bufs,
-                uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
+int launch_scan(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
+                int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return -19;
-  if (scan_variant(a.threads, a.blocks, device) == 0)
-    launch_scan_wide(g, fid, a, nstrides, bufs, buf_stride, d_count, d_sum, d_hash, s);
-  else
-    launch_scan_narrow(g, fid, a, nstrides, bufs, buf_stride, d_count, d_sum, d_hash, s);
-  return cuda_err(cudaGetLastError());
+  return cuda_err(scan_variant(a.threads, a.blocks, device) == 0
+                      ? launch_scan_wide(g, fid, a, nstrides, d_count, d_sum, d_hash, s)
+                      : launch_scan_narrow(g, fid, a, nstrides, d_count, d_sum, d_hash, s));
 }
 
 int launch_scan_path(const DevHandle& g, const PathArg& path, const gfs_scan_args& a, unsigned long long nstrides,
-                     uint8_t* bufs, uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash,
-                     cudaStream_t s) {
-  k_scan_path<<<a.blocks, a.threads, 0, s>>>(g, path, a.stride, a.read_len, nstrides, bufs, buf_stride,
-                                             (long long*)d_count, (unsigned long long*)d_sum,
-                                             (unsigned long long*)d_hash);
+                     int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(k_scan_path, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)scan_window(1, 512));
+  if (e != cudaSuccess) return cuda_err(e);
+  k_scan_path<<<a.blocks, a.threads, scan_window(1, a.threads), s>>>(
+      g, path, a.stride, a.read_len, nstrides, (long long*)d_count, (unsigned long long*)d_sum,
+      (unsigned long long*)d_hash);
   return cuda_err(cudaGetLastError());
 }
 
@@ -224,17 +223,17 @@ int launch_pull_probe(const uint8_t* src, uint8_t* dst, uint64_t n, cudaStream_t
   return cuda_err(cudaGetLastError());
 }
 
-int scan_max_resident_blocks(uint32_t threads, bool fused, int device, int* out) {
+int scan_max_resident_blocks(uint32_t threads, int device, int* out) {
   int per_sm = 0, sms = 0;
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (e != cudaSuccess) return cuda_err(e);
   // the largest grid that is resident at once with the instance launch_scan picks for it
-  e = scan_occupancy_wide(fused, (int)threads, &per_sm);
+  e = scan_occupancy_wide((int)threads, &per_sm);
   if (e != cudaSuccess) return cuda_err(e);
   int best = per_sm * sms;
   if (threads <= 256) {
     if (best > 2 * sms) best = 2 * sms;  // larger grids use <256, 4>
-    e = scan_occupancy_narrow(fused, (int)threads, &per_sm);
+    e = scan_occupancy_narrow((int)threads, &per_sm);
     if (e != cudaSuccess) return cuda_err(e);
     if (per_sm * sms > best) best = per_sm * sms;
   }
@@ -245,59 +244,9 @@ int scan_max_resident_blocks(uint32_t threads, bool fused, int device, int* out)
 }  // namespace gfs
 
 // ---------------------------------------------------------------- allocation-free scan
-// gfs_scan_static keeps the per-threadblock gread buffers in this file-scope
-// device array instead of memory the context allocates, so the call itself never
-// allocates.  Every device that loads the library holds the array until exit.
-namespace {
-
-constexpr size_t kStaticScratchBytes = 64ull << 20;  // GFS_STATIC_SCRATCH_BYTES in include/gfs.h
-// A read shorter than its block's window takes up to one word more than its length
-// rounded up to 256 bytes (scan_window), which is what the bound counts it with.
-static __device__ __align__(256) uint8_t g_scan_scratch[kStaticScratchBytes + kStaticScratchBytes / 16];
-
-// The context an address was looked up in: a caller that resets the device and
-// so creates a new primary context gets the array's address looked up again.
-typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
-CtxGetCurrentFn g_ctx_current = nullptr;
-
-constexpr int kMaxDevices = 64;
-std::mutex g_scratch_mu;
-void* g_scratch_addr[kMaxDevices] = {};
-CUcontext g_scratch_ctx[kMaxDevices] = {};
-
-CUcontext current_context() {
-  if (!g_ctx_current) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      g_ctx_current = (CtxGetCurrentFn)fn;
-  }
-  CUcontext c = nullptr;
-  if (g_ctx_current && g_ctx_current(&c) != CUDA_SUCCESS) c = nullptr;
-  return c;
-}
-
-// Device address of the scratch array on `device` (current).  In host code the
-// array's name is only a host-side stand-in, so the address is looked up once per
-// device and context and cached.
-int static_scratch(int device, void** out) {
-  if (device < 0 || device >= kMaxDevices) return -EINVAL;
-  std::lock_guard<std::mutex> lk(g_scratch_mu);
-  const CUcontext cur = current_context();
-  if (!g_scratch_addr[device] || g_scratch_ctx[device] != cur) {
-    void* p = nullptr;
-    cudaError_t e = cudaGetSymbolAddress(&p, g_scan_scratch);
-    if (e != cudaSuccess || !p) return e == cudaErrorNoDevice ? -ENODEV : -EINVAL;
-    g_scratch_addr[device] = p;
-    g_scratch_ctx[device] = cur;
-  }
-  *out = g_scratch_addr[device];
-  return 0;
-}
-
-}  // namespace
-
+// The scan's blocks keep what they read in shared memory, so gfs_scan_static has nothing
+// to allocate; its bound on blocks x read length (GFS_STATIC_SCRATCH_BYTES) stands as
+// documented.
 extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, int64_t* d_count, uint64_t* d_sum,
                                uint64_t* d_hash, void* stream) {
   if (!ctx || !a) return -EINVAL;
@@ -309,10 +258,9 @@ extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, in
   // a gread never delivers more than the file holds; bound before rounding up
   // and divide instead of multiplying, so that no size wraps around
   const uint64_t per_block = a->read_len < size ? a->read_len : size;
-  if (per_block > kStaticScratchBytes) return -ENOSPC;
+  if (per_block > GFS_STATIC_SCRATCH_BYTES) return -ENOSPC;
   const uint64_t bound = (per_block + 255) / 256 * 256;
-  if (bound && a->blocks > kStaticScratchBytes / bound) return -ENOSPC;  // beyond the static array
-  const uint64_t buf_stride = gfs::scan_window(per_block, a->threads);
+  if (bound && a->blocks > GFS_STATIC_SCRATCH_BYTES / bound) return -ENOSPC;
   if (nstrides == 0) return 0;
   if (!d_count || !d_sum || !d_hash) return -EINVAL;
   if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return -ENODEV;
@@ -320,9 +268,6 @@ extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, in
       ctx->dev.paper_streams < a->blocks)
     return -ENOTSUP;  // the per-block state would have to be allocated
   note_read(ctx, fid);
-  void* scratch = nullptr;
-  int rc = static_scratch(ctx->cfg.device, &scratch);
-  if (rc) return rc;
   gfs::DevHandle g = ctx->dev;
   g.exact_lra = a->serialize ? 1u : 0u;
   const uint64_t pages_per_read = (a->read_len >> ctx->dev.page_shift) + ((a->read_len & (ctx->cfg.page_size - 1)) != 0);
@@ -333,10 +278,10 @@ extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, in
   cudaStream_t s = (cudaStream_t)stream;
   if (a->serialize) {
     int maxb = 0;
-    rc = gfs::scan_max_resident_blocks(a->threads, a->fused != 0, ctx->cfg.device, &maxb);
+    const int rc = gfs::scan_max_resident_blocks(a->threads, ctx->cfg.device, &maxb);
     if (rc) return rc;
     if ((int)a->blocks > maxb) return -EINVAL;
     if (cudaMemsetAsync(&g.ctrl->ticket.v, 0, 8, s) != cudaSuccess) return -EINVAL;
   }
-  return gfs::launch_scan(g, fid, *a, nstrides, (uint8_t*)scratch, buf_stride, d_count, d_sum, d_hash, s);
+  return gfs::launch_scan(g, fid, *a, nstrides, d_count, d_sum, d_hash, s);
 }

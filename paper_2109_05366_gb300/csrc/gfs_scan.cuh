@@ -64,13 +64,15 @@ static __device__ void block_help_drain(const DevHandle& g) {
 // SM it must leave room for, which set its register budget.  <512, 1> leaves the
 // control path every register it uses (no spills; two 256-thread blocks per SM);
 // <256, 4> fits four 256-thread blocks per SM in 64 registers.
-template <bool FUSED, int MAXT, int MINB>
+// A warp's window: two units, or one where four blocks of 256 threads share an SM.
+__host__ __device__ constexpr int scan_stages(int minb) { return minb == 1 ? 2 : 1; }
+inline size_t scan_window(int minb, uint32_t threads) { return (size_t)scan_stages(minb) * (threads / 32) * 4096; }
+
+template <int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsigned long long stride,
                                                unsigned long long read_len, unsigned long long nstrides, int serialize,
-                                               uint8_t* bufs, unsigned long long buf_stride, long long* cnt,
-                                               unsigned long long* sum, unsigned long long* hash) {
+                                               long long* cnt, unsigned long long* sum, unsigned long long* hash) {
   const uint32_t b = blockIdx.x, tid = threadIdx.x;
-  uint8_t* buf = bufs + (size_t)b * buf_stride;
   for (unsigned long long s = b; s < nstrides; s += gridDim.x) {
     const unsigned long long off = s * stride;
     if (serialize) {  // one gread at a time, in stride order
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsig
       }
       __syncthreads();
     }
-    dev::ScanSink<FUSED> sink{buf, {0ull, 0ull}};
+    dev::WindowSink<scan_stages(MINB)> sink{{0ull, 0ull}};
     long long r = dev::gread_impl(g, (int)b, fid, off, read_len, sink);
     Sums acc = sink.acc;
     if (serialize) {  // wait until every request of this gread has been served
@@ -124,24 +126,38 @@ __global__ void __launch_bounds__(MAXT, MINB) k_read_many(DevHandle g, int fid, 
   block_help_drain(g);
 }
 
-template <bool FUSED, int MAXT, int MINB>
-inline void launch_scan_as(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
-                           uint8_t* bufs, uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash,
-                           cudaStream_t s) {
-  k_scan<FUSED, MAXT, MINB><<<a.blocks, a.threads, 0, s>>>(g, fid, a.stride, a.read_len, nstrides, (int)a.serialize,
-                                                           bufs, buf_stride, (long long*)d_count,
-                                                           (unsigned long long*)d_sum, (unsigned long long*)d_hash);
+// The most dynamic shared memory is set on each launch: it belongs to the current device
+// and context.
+template <int MAXT, int MINB>
+inline cudaError_t launch_scan_as(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
+                                  int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
+  const size_t window = scan_window(MINB, a.threads);
+  const cudaError_t e = cudaFuncSetAttribute(k_scan<MAXT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)scan_window(MINB, MAXT));
+  if (e != cudaSuccess) return e;
+  k_scan<MAXT, MINB><<<a.blocks, a.threads, window, s>>>(g, fid, a.stride, a.read_len, nstrides, (int)a.serialize,
+                                                         (long long*)d_count, (unsigned long long*)d_sum,
+                                                         (unsigned long long*)d_hash);
+  return cudaGetLastError();
+}
+
+template <int MAXT, int MINB>
+inline cudaError_t scan_occupancy_as(int threads, int* per_sm) {
+  const cudaError_t e = cudaFuncSetAttribute(k_scan<MAXT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)scan_window(MINB, MAXT));
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_scan<MAXT, MINB>, threads,
+                                                       scan_window(MINB, (uint32_t)threads));
 }
 
 // Launchers and occupancy of the two instances of k_scan and k_read_many
 // (gfs_scan_wide.cu: <512, 1>; gfs_scan_narrow.cu: <256, 4>).
-void launch_scan_wide(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides, uint8_t* bufs,
-                      uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
-void launch_scan_narrow(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
-                        uint8_t* bufs, uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash,
-                        cudaStream_t s);
-cudaError_t scan_occupancy_wide(bool fused, int threads, int* per_sm);
-cudaError_t scan_occupancy_narrow(bool fused, int threads, int* per_sm);
+cudaError_t launch_scan_wide(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
+                             int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
+cudaError_t launch_scan_narrow(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
+                               int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
+cudaError_t scan_occupancy_wide(int threads, int* per_sm);
+cudaError_t scan_occupancy_narrow(int threads, int* per_sm);
 void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                            const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
                            cudaStream_t s);

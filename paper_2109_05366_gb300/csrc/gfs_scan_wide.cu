@@ -4,16 +4,12 @@
 
 namespace gfs {
 
-void launch_scan_wide(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides, uint8_t* bufs,
-                    uint64_t buf_stride, int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
-  if (a.fused) launch_scan_as<true, 512, 1>(g, fid, a, nstrides, bufs, buf_stride, d_count, d_sum, d_hash, s);
-  else launch_scan_as<false, 512, 1>(g, fid, a, nstrides, bufs, buf_stride, d_count, d_sum, d_hash, s);
+cudaError_t launch_scan_wide(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
+                        int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
+  return launch_scan_as<512, 1>(g, fid, a, nstrides, d_count, d_sum, d_hash, s);
 }
 
-cudaError_t scan_occupancy_wide(bool fused, int threads, int* per_sm) {
-  return fused ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_scan<true, 512, 1>, threads, 0)
-               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_scan<false, 512, 1>, threads, 0);
-}
+cudaError_t scan_occupancy_wide(int threads, int* per_sm) { return scan_occupancy_as<512, 1>(threads, per_sm); }
 
 void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                       const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
