@@ -1960,16 +1960,21 @@ static __device__ void check_mark(const DevHandle& g, int stream, uint32_t fid, 
   if (m) async_readahead(g, stream, fid, fi, (unsigned long long)m - 1, w, seq0, deadline, s_frames);
 }
 
+// Count nbytes of a pinned page as delivered (one thread).  Returns whether that makes it
+// fully consumed, so that it goes to the consumed FIFO (per-threadblock LRA queues, Section
+// 5.1, keep none).  A page that already is fully consumed is not counted further: a count
+// that wrapped around after 4 GiB of reads of one cached page would queue it again and
+// again, until a push waits out its deadline on the full FIFO.
+static __device__ bool page_consume(const DevHandle& g, uint32_t f, uint32_t nbytes) {
+  const uint32_t v = ld_rlx(&g.fvalid[f]);
+  if (ld_rlx(&g.fconsumed[f]) >= v) return false;
+  const uint32_t c = atomicAdd(&g.fconsumed[f], nbytes);
+  return g.repl != GFS_REPL_TB_LRA && c < v && c + nbytes >= v;
+}
+
 // R5: account the delivered bytes, unpin, and queue the frame once fully consumed.
 static __device__ void release_page(const DevHandle& g, int f, uint32_t nbytes, unsigned long long deadline) {  // one thread
-  if (g.repl == GFS_REPL_TB_LRA) {  // per-threadblock LRA queues (Section 5.1) replace the consumed FIFO
-    atomicAdd(&g.fconsumed[f], nbytes);  // nothing waits for the old count
-    frame_unpin(g, f);
-    return;
-  }
-  uint32_t c = atomicAdd(&g.fconsumed[f], nbytes);
-  uint32_t v = ld_rlx(&g.fvalid[f]);
-  bool push = c < v && c + nbytes >= v;
+  const bool push = page_consume(g, (uint32_t)f, nbytes);
   frame_unpin(g, f);
   if (push) fifo_push(g, (uint32_t)f, deadline);
 }
@@ -2045,11 +2050,7 @@ static __device__ bool run_consume(const DevHandle& g, uint32_t f, unsigned long
   const unsigned long long base = q << g.page_shift;
   const unsigned long long lo = off > base ? off : base;
   const unsigned long long hi = end < base + g.page_size ? end : base + g.page_size;
-  const uint32_t nb = (uint32_t)(hi - lo);
-  const uint32_t c = atomicAdd(&g.fconsumed[f], nb);
-  if (g.repl == GFS_REPL_TB_LRA) return false;  // per-threadblock LRA queues keep no consumed FIFO
-  const uint32_t v = ld_rlx(&g.fvalid[f]);
-  return c < v && c + nb >= v;
+  return page_consume(g, f, (uint32_t)(hi - lo));
 }
 
 // Whole block, after it read the run: R5 for its n pages (page p + i in frame
@@ -2864,10 +2865,15 @@ static __device__ __forceinline__ uint32_t read_batch(const DevHandle& g, const 
         }
       }
     }
-    uint32_t c = 0, v = 0;
-    if (mine && (int)lane == lead) c = atomicAdd(&g.fconsumed[f], all);
-    c = __shfl_sync(kFull, c, lead) + before;
-    if (mine) v = ld_rlx(&g.fvalid[f]);
+    uint32_t c = 0;
+    const uint32_t v = mine ? ld_rlx(&g.fvalid[f]) : 0u;
+    if (mine && (int)lane == lead) {  // as page_consume
+      c = ld_rlx(&g.fconsumed[f]);
+      if (c < v) c = atomicAdd(&g.fconsumed[f], all);
+      else c = v;
+    }
+    c = __shfl_sync(kFull, c, lead);
+    if (c < v) c += before;
     const bool push = mine && g.repl != GFS_REPL_TB_LRA && c < v && c + nb >= v;
     __threadfence();
     if (mine && (int)lane == lead) atomicSub(&g.fpins[f], (uint32_t)__popc(peers));

@@ -120,3 +120,25 @@ def test_batches_of_many_blocks_share_pages(torch_cuda, gfs, datadir, frames):
         assert ret[i] == len(part)
         assert np.array_equal(buf[d[i]:d[i] + len(part)], part)
     assert st["greads"] == n and st["timeouts"] == 0
+
+
+@pytest.mark.parametrize("lat", [0, 16])
+def test_a_cached_page_read_over_and_over_is_queued_once(torch_cuda, gfs, datadir, lat):
+    """4 GiB of reads of a page and more must not count it as newly consumed again."""
+    torch = torch_cuda
+    page, n, passes = 4 * KiB, 1 << 17, 80  # 2^32 bytes are eight passes
+    path = os.path.join(datadir, "batches_wrap.bin")
+    np.random.default_rng(15).integers(0, 256, page, dtype=np.uint8).tofile(path)
+    with gfs.Context(cache_bytes=4 * page, page_size=page, latency_capacity=lat, timeout_ns=200_000_000) as ctx:
+        fid = ctx.open(path)
+        ctx.fadvise(fid, gfs.ADV_RANDOM)
+        off = torch.zeros(n, dtype=torch.int64, device="cuda")
+        buf = torch.zeros(n * page, dtype=torch.uint8, device="cuda")
+        ret = torch.zeros(n, dtype=torch.int64, device="cuda")
+        dst = torch.arange(n, dtype=torch.int64, device="cuda") * page
+        for _ in range(passes):
+            ctx.read_many(fid, off, torch.full_like(off, page), dst, buf, ret, blocks=608, threads=128)
+        torch.cuda.synchronize()
+        st = ctx.stats()
+    assert st["timeouts"] == 0 and st["evictions"] == 0
+    assert st["hits"] + st["misses"] >= n * passes and (ret == page).all()
