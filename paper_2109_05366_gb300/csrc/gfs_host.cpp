@@ -673,6 +673,8 @@ int gfs_init(const gfs_config* cfg_in, gfs_ctx** out) {
   int rc = load_driver_fns();
   if (rc) return rc;
   CK(cudaSetDevice(c.device));
+  rc = scan_setup();
+  if (rc) return rc;
 
   gfs_ctx* ctx = new (std::nothrow) gfs_ctx();
   if (!ctx) return -ENOMEM;

@@ -49,6 +49,7 @@ struct HostFile {
 class IoService;
 
 // Entry points of the device code, implemented in gfs_kernels.cu.
+int scan_setup();  // shared memory of the scan kernels on the current device; before their first launch
 int launch_reset(const DevHandle& g, cudaStream_t s);
 int launch_drain(const DevHandle& g, cudaStream_t s);
 int launch_scan(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,

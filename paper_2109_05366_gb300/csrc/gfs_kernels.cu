@@ -148,6 +148,14 @@ static int cuda_err(cudaError_t e) {
   return -22;
 }
 
+int scan_setup() {
+  cudaError_t e = scan_setup_wide();
+  if (e == cudaSuccess) e = scan_setup_narrow();
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_scan_path, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)scan_window(1, 512));
+  return cuda_err(e);
+}
+
 int launch_reset(const DevHandle& g, cudaStream_t s) {
   k_reset<<<304, 512, 0, s>>>(g);
   return cuda_err(cudaGetLastError());
@@ -182,9 +190,6 @@ int launch_scan(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned lo
 
 int launch_scan_path(const DevHandle& g, const PathArg& path, const gfs_scan_args& a, unsigned long long nstrides,
                      int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
-  const cudaError_t e = cudaFuncSetAttribute(k_scan_path, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)scan_window(1, 512));
-  if (e != cudaSuccess) return cuda_err(e);
   k_scan_path<<<a.blocks, a.threads, scan_window(1, a.threads), s>>>(
       g, path, a.stride, a.read_len, nstrides, (long long*)d_count, (unsigned long long*)d_sum,
       (unsigned long long*)d_hash);

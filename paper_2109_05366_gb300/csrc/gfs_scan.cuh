@@ -126,15 +126,12 @@ __global__ void __launch_bounds__(MAXT, MINB) k_read_many(DevHandle g, int fid, 
   block_help_drain(g);
 }
 
-// The most dynamic shared memory is set on each launch: it belongs to the current device
-// and context.
+// gfs_init sets the most dynamic shared memory of the instances (scan_setup): on each
+// launch that took as long as a fifth of a 10 us call.
 template <int MAXT, int MINB>
 inline cudaError_t launch_scan_as(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
                                   int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s) {
   const size_t window = scan_window(MINB, a.threads);
-  const cudaError_t e = cudaFuncSetAttribute(k_scan<MAXT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)scan_window(MINB, MAXT));
-  if (e != cudaSuccess) return e;
   k_scan<MAXT, MINB><<<a.blocks, a.threads, window, s>>>(g, fid, a.stride, a.read_len, nstrides, (int)a.serialize,
                                                          (long long*)d_count, (unsigned long long*)d_sum,
                                                          (unsigned long long*)d_hash);
@@ -142,10 +139,13 @@ inline cudaError_t launch_scan_as(const DevHandle& g, int fid, const gfs_scan_ar
 }
 
 template <int MAXT, int MINB>
+inline cudaError_t scan_setup_as() {
+  return cudaFuncSetAttribute(k_scan<MAXT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)scan_window(MINB, MAXT));
+}
+
+template <int MAXT, int MINB>
 inline cudaError_t scan_occupancy_as(int threads, int* per_sm) {
-  const cudaError_t e = cudaFuncSetAttribute(k_scan<MAXT, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)scan_window(MINB, MAXT));
-  if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_scan<MAXT, MINB>, threads,
                                                        scan_window(MINB, (uint32_t)threads));
 }
@@ -156,6 +156,8 @@ cudaError_t launch_scan_wide(const DevHandle& g, int fid, const gfs_scan_args& a
                              int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
 cudaError_t launch_scan_narrow(const DevHandle& g, int fid, const gfs_scan_args& a, unsigned long long nstrides,
                                int64_t* d_count, uint64_t* d_sum, uint64_t* d_hash, cudaStream_t s);
+cudaError_t scan_setup_wide();
+cudaError_t scan_setup_narrow();
 cudaError_t scan_occupancy_wide(int threads, int* per_sm);
 cudaError_t scan_occupancy_narrow(int threads, int* per_sm);
 void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,

@@ -9,6 +9,8 @@ cudaError_t launch_scan_narrow(const DevHandle& g, int fid, const gfs_scan_args&
   return launch_scan_as<256, 4>(g, fid, a, nstrides, d_count, d_sum, d_hash, s);
 }
 
+cudaError_t scan_setup_narrow() { return scan_setup_as<256, 4>(); }
+
 cudaError_t scan_occupancy_narrow(int threads, int* per_sm) { return scan_occupancy_as<256, 4>(threads, per_sm); }
 
 void launch_read_many_narrow(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,

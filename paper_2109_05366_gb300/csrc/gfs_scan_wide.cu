@@ -9,6 +9,8 @@ cudaError_t launch_scan_wide(const DevHandle& g, int fid, const gfs_scan_args& a
   return launch_scan_as<512, 1>(g, fid, a, nstrides, d_count, d_sum, d_hash, s);
 }
 
+cudaError_t scan_setup_wide() { return scan_setup_as<512, 1>(); }
+
 cudaError_t scan_occupancy_wide(int threads, int* per_sm) { return scan_occupancy_as<512, 1>(threads, per_sm); }
 
 void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
