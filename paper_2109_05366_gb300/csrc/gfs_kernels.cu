@@ -207,7 +207,7 @@ int launch_read_many(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return -19;
   if (scan_variant(threads, blocks, device) == 0)
-    launch_read_many_wide(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, s);
+    launch_read_many_wide(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, cold, s);
   else
     launch_read_many_narrow(g, fid, n, d_off, d_len, d_dst, d_buf, d_ret, blocks, threads, cold, s);
   return cuda_err(cudaGetLastError());

@@ -109,8 +109,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsig
 // Independent greads (Section 2.2): block b serves reads b, b + B, ... of the
 // list.  MAXT, MINB as for k_scan: a small read costs a block mostly control-path
 // latency, so the reads in flight grow with the blocks resident per SM.
-// BATCH: reads of cached pages go in batches.  The <256, 4> instance also exists without,
-// for lists on files of which nothing can be cached yet: there the batches' call makes the
+// BATCH: reads of cached pages go in batches.  Both instances also exist without, for lists on files of which nothing can be cached yet: there the batches' call makes the
 // register allocator spill what gread holds (131072 random 4 KiB pages from the host:
 // 2337 us with, 2223 us without).
 template <bool BATCH, int MAXT, int MINB>
@@ -162,7 +161,7 @@ cudaError_t scan_occupancy_wide(int threads, int* per_sm);
 cudaError_t scan_occupancy_narrow(int threads, int* per_sm);
 void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                            const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
-                           cudaStream_t s);
+                           bool cold, cudaStream_t s);
 void launch_read_many_narrow(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                              const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
                              bool cold, cudaStream_t s);

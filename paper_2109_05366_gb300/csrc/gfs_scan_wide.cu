@@ -15,9 +15,10 @@ cudaError_t scan_occupancy_wide(int threads, int* per_sm) { return scan_occupanc
 
 void launch_read_many_wide(const DevHandle& g, int fid, uint32_t n, const uint64_t* d_off, const uint64_t* d_len,
                       const uint64_t* d_dst, uint8_t* d_buf, int64_t* d_ret, uint32_t blocks, uint32_t threads,
-                      cudaStream_t s) {
-  k_read_many<true, 512, 1><<<blocks, threads, 0, s>>>(
-      g, fid, dev::ReadList{d_off, d_len, d_dst, d_buf, (long long*)d_ret, n});
+                      bool cold, cudaStream_t s) {
+  const dev::ReadList list{d_off, d_len, d_dst, d_buf, (long long*)d_ret, n};
+  if (cold) k_read_many<false, 512, 1><<<blocks, threads, 0, s>>>(g, fid, list);
+  else k_read_many<true, 512, 1><<<blocks, threads, 0, s>>>(g, fid, list);
 }
 
 }  // namespace gfs
