@@ -2496,12 +2496,14 @@ __device__ __noinline__ long long read_run(const DevHandle& g, uint32_t fid, uns
 
 // Whole block: copy the pages of the pending self-served request (frames in
 // frames[0 .. n), pages page_lo ..) from the file's mapping into their frames and
-// publish them READY.  No-op when none is pending.  Block-uniform.
-__device__ __forceinline__ void block_self_serve(const DevHandle& g, unsigned long long dev_map,
+// publish them READY.  n: the pending request's pages, read where a barrier stands
+// between the read and the next store to self_job() (warp 0 goes on to check_mark, which
+// may leave the next request, while other warps are still on their way here); 0: none
+// pending, no-op.  Block-uniform.
+__device__ __forceinline__ void block_self_serve(const DevHandle& g, uint32_t n, unsigned long long dev_map,
                                                  const uint32_t* frames) {
-  SelfJob& j = self_job();
-  const uint32_t n = j.n;
   if (n == 0) return;
+  SelfJob& j = self_job();
   const unsigned long long p0 = j.page_lo;
   const uint32_t tid = threadIdx.x, nt = blockDim.x;
   const bool small = g.page_size <= (16u << 10);  // small pages: a warp per page, many in flight
@@ -2532,13 +2534,12 @@ __device__ __forceinline__ void block_self_serve(const DevHandle& g, unsigned lo
 // 64 MiB by 64 blocks 445 us, now 412 us.
 constexpr uint32_t kServeChunk = 128u << 10;
 template <class Sink>
-static __device__ __noinline__ uint32_t block_serve_arriving(const DevHandle& g, unsigned long long dev_map,
-                                                             const uint32_t* frames, unsigned long long off,
-                                                             unsigned long long end, Sink& sink,
-                                                             unsigned long long deadline) {
-  SelfJob& j = self_job();
-  const uint32_t n = j.n;
+static __device__ __noinline__ uint32_t block_serve_arriving(const DevHandle& g, uint32_t n,
+                                                             unsigned long long dev_map, const uint32_t* frames,
+                                                             unsigned long long off, unsigned long long end,
+                                                             Sink& sink, unsigned long long deadline) {
   if (n == 0) return 0;
+  SelfJob& j = self_job();
   const unsigned long long p0 = j.page_lo;
   const uint32_t tid = threadIdx.x, nt = blockDim.x;
   const uint32_t mine = j.demand < n ? j.demand : n;
@@ -2638,13 +2639,14 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
     const int f = s_frame;
     int st = s_state;
     const PaperJob job = s_job;
+    const uint32_t pending = self_job().n;
     __syncthreads();
     // the request the miss just made, when its pages are the block's to copy
     uint32_t took = 0;
     if (Sink::kArrive && g.page_size > (16u << 10))
-      took = block_serve_arriving(g, fi.dev_map, s_frames, off, end, sink, deadline);
+      took = block_serve_arriving(g, pending, fi.dev_map, s_frames, off, end, sink, deadline);
     else
-      block_self_serve(g, fi.dev_map, s_frames);
+      block_self_serve(g, pending, fi.dev_map, s_frames);
     if (f < 0) {
       err = f;
       break;
@@ -2666,7 +2668,7 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
     }
     if (tid < 32) check_mark(g, stream, (uint32_t)fid, fi, f, seq0, deadline, s_frames);
     __syncthreads();
-    block_self_serve(g, fi.dev_map, s_frames);  // the asynchronous window check_mark requested, if any
+    block_self_serve(g, self_job().n, fi.dev_map, s_frames);  // the asynchronous window check_mark requested, if any
     const unsigned long long base = p << g.page_shift;
     const unsigned long long lo = off > base ? off : base;
     const unsigned long long hi = end < base + g.page_size ? end : base + g.page_size;
