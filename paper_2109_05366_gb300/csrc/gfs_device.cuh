@@ -1864,9 +1864,12 @@ static __device__ int block_paper_job(const DevHandle& g, int stream, uint32_t f
 }
 
 // Find or install page p and pin its frame for the caller (warp 0); does not
-// wait.  Returns the frame (its state in *state) or -errno.
+// wait.  absent: a look-up has just found that p is not in the cache, so that the
+// first one here is spared.  Returns the frame or -errno; *state is its state, with
+// kMissed where this call installed it.
+constexpr int kMissed = 0x100;
 static __device__ int acquire_begin(const DevHandle& g, int stream, uint32_t fid, const FileDev& fi, unsigned long long p,
-                             unsigned long long p1, unsigned long long seq0, unsigned long long deadline,
+                             unsigned long long p1, bool absent, unsigned long long seq0, unsigned long long deadline,
                              uint32_t* s_frames, int* state, PaperJob* job) {
   const int lane = lane_id();
   const unsigned long long key = make_key(fid, p);
@@ -1877,7 +1880,8 @@ static __device__ int acquire_begin(const DevHandle& g, int stream, uint32_t fid
       if (lane == 0) stat_add(g, ST_TIMEOUTS, 1);
       return -kETIMEDOUT;
     }
-    int f = tab_lookup(g, key);
+    int f = absent ? -1 : tab_lookup(g, key);
+    absent = false;  // a page that someone else inserts meanwhile comes back as -EAGAIN
     if (f >= 0) {
       int st = -1;
       if (lane == 0) {
@@ -1902,7 +1906,7 @@ static __device__ int acquire_begin(const DevHandle& g, int stream, uint32_t fid
       continue;
     }
     if (r < 0) return r;
-    *state = FR_FILLING;
+    *state = FR_FILLING | kMissed;
     return r;
   }
 }
@@ -1995,13 +1999,15 @@ constexpr uint32_t kRunWarps = 16;  // warps that look pages up (the widest bloc
 constexpr uint32_t kRunPages = 32 * kRunWarps;
 
 // Warp: look up and pin pages p .. p + k - 1 (k <= 32).  Returns the length of
-// the leading run of pages that are READY without a mark, FILLING or COPYING;
-// their frames are left in s_f, pinned, and the mask of those not READY yet in
-// *wait.  Pages after the run are left unpinned.
-static __device__ uint32_t run_begin(const DevHandle& g, uint32_t fid, unsigned long long p, uint32_t k, bool marks,
+// the leading run of pages that are READY without a mark, FILLING or COPYING, or -1
+// where page p is not in the cache at all; their frames are left in s_f, pinned, and
+// the mask of those not READY yet in *wait.  Pages after the run are left unpinned.
+static __device__ int run_begin(const DevHandle& g, uint32_t fid, unsigned long long p, uint32_t k, bool marks,
                                      uint32_t* s_f, uint32_t* wait) {
   const int lane = lane_id();
   int f = -1;  // frame of page p + lane
+  uint32_t ovf = 0;  // page p's home bucket overflowed; in flight with the bucket
+  if (lane == 0) ovf = ld_rlx(&g.tovf[bucket_of(make_key(fid, p), g.nbuckets)]);
   // home buckets only, eight keys in flight: a key in an overflow bucket ends the run
   for (uint32_t q0 = 0; q0 < k; q0 += 8) {
     unsigned long long e[8];
@@ -2020,6 +2026,12 @@ static __device__ uint32_t run_begin(const DevHandle& g, uint32_t fid, unsigned 
       gap |= q0 + j < k && fj < 0;
     }
     if (gap) break;
+  }
+  // page p is not here: nothing to pin, and no fence
+  const int f0 = bcast(f);
+  if (f0 < 0) {
+    if (lane == 0) *wait = 0;
+    return bcast((int)ovf) ? 0 : -1;
   }
   // pin as frame_pin does, one lane per page
   const bool mine = (uint32_t)lane < k && f >= 0;
@@ -2040,7 +2052,7 @@ static __device__ uint32_t run_begin(const DevHandle& g, uint32_t fid, unsigned 
   if ((uint32_t)lane < c) s_f[lane] = (uint32_t)f;
   if (lane == 0) *wait = wm;
   __syncwarp();
-  return c;
+  return (int)c;
 }
 
 // One lane, one page of a run (frame f, page q; the gread covers [off, end)): R5's
@@ -2424,8 +2436,10 @@ struct WindowSink {
 // Whole block: read the run of cached pages that starts at page p (p1 = last
 // page of the gread, which covers [off, end)): pin it, wait for pages still being
 // filled in page order, hand it to the sink, release it.  Returns the number of
-// pages read (0: page p takes the one-page path) or -errno.
+// pages read (0: page p takes the one-page path; kAbsent: it does, and it is not in
+// the cache) or -errno.
 // Kept out of line so that it leaves the one-page path's registers alone.
+constexpr long long kAbsent = 1ll << 32;
 template <class Sink>
 __device__ __noinline__ long long read_run(const DevHandle& g, uint32_t fid, unsigned long long p,
                                            unsigned long long p1, unsigned long long off, unsigned long long end,
@@ -2438,10 +2452,16 @@ __device__ __noinline__ long long read_run(const DevHandle& g, uint32_t fid, uns
   const uint32_t want = left < 32u * nw ? (uint32_t)left : 32u * nw;  // pages looked up
   uint32_t c = 0;                                                   // this warp's leading pages
   if (32 * w < want) {
-    c = run_begin(g, fid, p + 32 * w, want - 32 * w < 32 ? want - 32 * w : 32, marks, s_rf + 32 * w, &s_rwait[w]);
-    if ((tid & 31) == 0) s_rn[w] = c;
+    const int r =
+        run_begin(g, fid, p + 32 * w, want - 32 * w < 32 ? want - 32 * w : 32, marks, s_rf + 32 * w, &s_rwait[w]);
+    c = r < 0 ? 0u : (uint32_t)r;
+    if ((tid & 31) == 0) s_rn[w] = w == 0 ? (uint32_t)r : c;
   }
   __syncthreads();
+  if (s_rn[0] == ~0u) {
+    if (w && (tid & 31) < c) atomicSub(&g.fpins[s_rf[tid]], 1u);
+    return kAbsent;
+  }
   uint32_t n = 0, rw = 0;  // the run; the warps that hold it
   while (32 * rw < want) {
     n += s_rn[rw];
@@ -2479,10 +2499,7 @@ __device__ __noinline__ long long read_run(const DevHandle& g, uint32_t fid, uns
       ++waited;
     }
   }
-  if (n == 0) {
-    __syncthreads();
-    return 0;
-  }
+  if (n == 0) return 0;
   if (tid == 0) {
     stat_add(g, ST_HITS, n);
     stat_add(g, ST_COALESCED, waited);
@@ -2602,21 +2619,31 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
   if (off >= fi.size || len == 0) return 0;
   const unsigned long long end = (len > fi.size - off) ? fi.size : off + len;
   const unsigned long long p0 = off >> g.page_shift, p1 = (end - 1) >> g.page_shift;
-  if (tid == 0) s_seq0 = (seq << kOwnerBits) | owner_of(stream);
+  if (tid == 0) {
+    s_seq0 = (seq << kOwnerBits) | owner_of(stream);
+    s_state = 0;
+  }
   __syncthreads();
   const unsigned long long seq0 = s_seq0;
   const unsigned long long deadline = now_ns() + g.timeout_ns;
   long long err = 0;
   const bool runs = g.mode != GFS_MODE_PAPER && p1 > p0;
   const bool marks = g.mode == GFS_MODE_READAHEAD && g.async_ra && fi.ra;
+  const bool alone = !(g.mode == GFS_MODE_READAHEAD && fi.ra);  // a miss requests its own page only
   for (unsigned long long p = p0; p <= p1;) {
-    if (runs) {
+    bool absent = false;
+    // After a miss of one page the next is most likely not here either: no run is looked
+    // for.  A look-up for a run that fails costs 1 to 2 us: an on-demand scan of 16 MiB of
+    // cold 4 KiB pages by 16 blocks took 3600 us with one at each page, 3042 us so (64 KiB
+    // pages: 348 and 323 us).
+    if (runs && !(alone && (s_state & kMissed))) {
       const long long n = read_run(g, (uint32_t)fid, p, p1, off, end, sink, marks, deadline);
       if (n < 0) {
         err = n;
         break;
       }
-      if (n) {
+      absent = n == kAbsent;
+      if (n && !absent) {
         p += (unsigned long long)n;
         continue;
       }
@@ -2628,7 +2655,7 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
     __syncthreads();
     if (tid < 32) {
       int st = 0;
-      int r = acquire_begin(g, stream, (uint32_t)fid, fi, p, p1, seq0, deadline, s_frames, &st, &s_job);
+      int r = acquire_begin(g, stream, (uint32_t)fid, fi, p, p1, absent, seq0, deadline, s_frames, &st, &s_job);
       if (tid == 0) {
         s_frame = r;
         s_one = (uint32_t)r;
@@ -2637,7 +2664,7 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
     }
     __syncthreads();
     const int f = s_frame;
-    int st = s_state;
+    int st = s_state & ~kMissed;
     const PaperJob job = s_job;
     const uint32_t pending = self_job().n;
     __syncthreads();
