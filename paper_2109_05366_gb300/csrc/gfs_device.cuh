@@ -2251,10 +2251,14 @@ __device__ __forceinline__ const uint8_t* run_at(const DevHandle& g, const RunVi
   return g.frames + ((size_t)r.f[rel >> g.page_shift] << g.page_shift) + ((uint32_t)rel & (g.page_size - 1u));
 }
 
+// Bytes of a page that arrives from the host a sink is given at a time (a multiple of 16).
+constexpr uint32_t kPiece = 128u << 10;
+
 // The gread into a user buffer: the byte at offset off goes to buf[0].  A warp takes a
 // unit of a page at a time.
 struct BufferSink {
   static constexpr bool kArrive = false;  // the reads of the 64-register instance are bound by their control path
+  __device__ __forceinline__ uint32_t piece() const { return kPiece; }
   uint8_t* buf;
   unsigned long long off;
   __device__ __noinline__ void take(const DevHandle& g, const RunView& r) {
@@ -2346,6 +2350,7 @@ __device__ __forceinline__ void unit_sums(Sums& acc, const uint4* v, unsigned lo
 // to a buffer per block and 445 us in place.
 struct SumSink {
   static constexpr bool kArrive = true;
+  __device__ __forceinline__ uint32_t piece() const { return kPiece; }
   Sums acc;
   __device__ __noinline__ void take(const DevHandle& g, const RunView& r) {
     const uint32_t w = threadIdx.x >> 5, nw = blockDim.x >> 5, units = run_units(r);
@@ -2381,6 +2386,7 @@ __device__ __forceinline__ void async_word(uint32_t to, const uint8_t* from) {
 template <int STAGES>
 struct WindowSink {
   static constexpr bool kArrive = true;
+  __device__ __forceinline__ uint32_t piece() const { return kPiece; }
   Sums acc;
 
   // Start copying the unit at file offset `at` into the lane's words of a cell.
@@ -2539,62 +2545,99 @@ __device__ __forceinline__ void block_self_serve(const DevHandle& g, uint32_t n,
 }
 
 // The same for pages above 16 KiB and a sink that takes bytes as they arrive
-// (Sink::kArrive): each page is published as soon as it is copied, and the leading
-// pages of the request that the gread [off, end) itself asked for are handed to its
-// sink kServeChunk bytes at a time as they arrive, before they are published: a page
-// that is FILLING cannot be evicted, so it needs no pin for that.  They are accounted
-// as if read afterwards, in page order.  Returns how many pages were delivered so (0
-// where none is pending).  Block-uniform.
+// (Sink::kArrive): the leading pages of the request that the gread [off, end) itself
+// asked for are handed to its sink.  Pages that it wants whole go there Sink::piece()
+// bytes at a time as they arrive, pages smaller than that several at a time, before they
+// are published: a page that is FILLING cannot be evicted, so it needs no pin for that.
+// Of a page that it wants in part, other greads are likely to want and await the rest:
+// such pages are copied first and published, pinned, before the sink takes any (1 MiB in
+// one page that 16 blocks share: 110 us with pieces, 105 us so).  The pages are accounted
+// in page order.  Returns how many pages were delivered (0 where none is
+// pending).  Block-uniform.
 // Bound by the host link.  With the copy of the whole request first and the consumer
 // after it, the blocks of a first pass all copied at the same time and then all
 // consumed while the link idled: histogram of 256 MiB 1602 us, now 1452 us; scan of
 // 64 MiB by 64 blocks 445 us, now 412 us.
-constexpr uint32_t kServeChunk = 128u << 10;
 template <class Sink>
-static __device__ __noinline__ uint32_t block_serve_arriving(const DevHandle& g, uint32_t n,
-                                                             unsigned long long dev_map, const uint32_t* frames,
-                                                             unsigned long long off, unsigned long long end,
-                                                             Sink& sink, unsigned long long deadline) {
+static __device__ __noinline__ uint32_t block_serve_arriving(const DevHandle& g, uint32_t n, const FileDev& fi,
+                                                             const uint32_t* frames, unsigned long long off,
+                                                             unsigned long long end, Sink& sink,
+                                                             unsigned long long deadline) {
   if (n == 0) return 0;
   SelfJob& j = self_job();
   const unsigned long long p0 = j.page_lo;
   const uint32_t tid = threadIdx.x, nt = blockDim.x;
   const uint32_t mine = j.demand < n ? j.demand : n;
-  for (uint32_t i = 0; i < n; ++i) {
-    const uint32_t f = frames[i], valid = ld_rlx(&g.fvalid[f]);
+  // whether the gread wants a part of page i only (the first or the last of its pages)
+  const auto part = [&](uint32_t i) {
     const unsigned long long base = (p0 + i) << g.page_shift;
-    const unsigned long long lo = off > base ? off : base;
-    const unsigned long long hi = end < base + valid ? end : base + valid;
-    const uint8_t* src = (const uint8_t*)(dev_map + base);
-    uint8_t* dst = g.frames + ((size_t)f << g.page_shift);
-    if (i >= mine) {
-      copy_in(src, dst, valid, tid, nt);
-    } else {
-      for (uint32_t c = 0; c < valid; c += kServeChunk) {
-        const uint32_t m = valid - c < kServeChunk ? valid - c : kServeChunk;
-        copy_in(src + c, dst + c, m, tid, nt);
-        const unsigned long long a = lo > base + c ? lo : base + c, b = hi < base + c + m ? hi : base + c + m;
-        if (a < b) {
+    return off > base || end < base + expected_valid(g, fi, p0 + i);
+  };
+  const auto fetch = [&](uint32_t i, uint32_t c, uint32_t m) {
+    copy_in((const uint8_t*)(fi.dev_map + ((p0 + i) << g.page_shift) + c),
+            g.frames + ((size_t)frames[i] << g.page_shift) + c, m, tid, nt);
+  };
+  const bool head = part(0), tail = mine > 1 && part(mine - 1);
+  if (head) fetch(0, 0, expected_valid(g, fi, p0));
+  if (tail) fetch(mine - 1, 0, expected_valid(g, fi, p0 + mine - 1));
+  if (head || tail) {
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      if (tail) atomicAdd(&g.fpins[frames[mine - 1]], 1u);  // the first page has the miss's pin
+      if (head) st_rel(&g.fstate[frames[0]], FR_READY);
+      if (tail) st_rel(&g.fstate[frames[mine - 1]], FR_READY);
+    }
+  }
+  const unsigned long long piece = sink.piece();
+  for (uint32_t i = 0; i < mine;) {
+    const unsigned long long base = (p0 + i) << g.page_shift;
+    if (part(i)) {
+      const unsigned long long lim = base + expected_valid(g, fi, p0 + i);
+      const unsigned long long lo = off > base ? off : base, hi = end < lim ? end : lim;
+      sink.take(g, RunView{frames + i, p0 + i, lo, hi});
+      __syncthreads();
+      if (tid == 0) release_page(g, (int)frames[i], (uint32_t)(hi - lo), deadline);
+      ++i;
+      continue;
+    }
+    uint32_t k = 1;  // pages i .. i + k - 1 in one piece or (k = 1) page i in several
+    while (i + k < mine && (unsigned long long)(k + 1) << g.page_shift <= piece && !part(i + k)) ++k;
+    for (uint32_t x = i; x < i + k; ++x) {
+      const uint32_t valid = expected_valid(g, fi, p0 + x);
+      for (uint32_t c = 0; c < valid;) {
+        const uint32_t m = valid - c < piece ? valid - c : (uint32_t)piece;
+        fetch(x, c, m);
+        c += m;
+        if (x + 1 == i + k) {
+          const unsigned long long to = ((p0 + x) << g.page_shift) + c;
           __syncthreads();
-          sink.take(g, RunView{frames + i, p0 + i, a, b});
+          sink.take(g, RunView{frames + i, p0 + i, k > 1 ? base : to - m, to});
         }
       }
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) {
-      // counted before the page can be evicted, queued once it can
-      const bool push = i < mine && run_consume(g, f, p0 + i, off, end);
-      st_rel(&g.fstate[f], FR_READY);
-      if (i == 0 && mine) frame_unpin(g, (int)f);  // the page that missed
-      if (push) fifo_push(g, f, deadline);
-    }
+    if (tid == 0)
+      for (uint32_t x = i; x < i + k; ++x) {
+        // R5 for a page nobody else has read yet, as one store; it cannot be evicted before
+        // it is READY, so the pin of the page that missed goes first and needs no fence
+        const uint32_t f = frames[x];
+        st_rlx(&g.fconsumed[f], expected_valid(g, fi, p0 + x));
+        if (x == 0) atomicSub(&g.fpins[f], 1u);
+        st_rel(&g.fstate[f], FR_READY);
+        if (g.repl != GFS_REPL_TB_LRA) fifo_push(g, f, deadline);
+      }
+    i += k;
+  }
+  for (uint32_t i = mine; i < n; ++i) {  // readahead
+    fetch(i, 0, expected_valid(g, fi, p0 + i));
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) st_rel(&g.fstate[frames[i]], FR_READY);
   }
   if (tid == 0 && mine > 1) stat_add(g, ST_HITS, mine - 1);
-  __syncthreads();
-  if (tid == 0) j.n = 0;
-  __syncthreads();
-  return mine;
+  return mine;  // gread clears the request before the next one, behind a barrier
 }
 
 // Threadblock-collective read of [off, off + len) of file `fid` into a sink.
@@ -2671,7 +2714,7 @@ __device__ long long gread_impl(const DevHandle& g, int stream, int fid, unsigne
     // the request the miss just made, when its pages are the block's to copy
     uint32_t took = 0;
     if (Sink::kArrive && g.page_size > (16u << 10))
-      took = block_serve_arriving(g, pending, fi.dev_map, s_frames, off, end, sink, deadline);
+      took = block_serve_arriving(g, pending, fi, s_frames, off, end, sink, deadline);
     else
       block_self_serve(g, pending, fi.dev_map, s_frames);
     if (f < 0) {
