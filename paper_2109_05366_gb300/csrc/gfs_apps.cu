@@ -31,6 +31,7 @@ constexpr uint32_t kSmemBins = 8192;  // histogram bins kept in shared memory (t
 // shared memory: 130.  Checksums kept by row, with one 64-bit multiply-add a word: 152,
 // a serial chain.)
 struct RowdotSink {
+  static constexpr bool kFar = false;
   static constexpr bool kArrive = true;
   // A row for every warp: with pieces of fewer rows most warps wait (first pass over a 2000 x
   // 8192 matrix in 64 KiB pages: 723 us in pieces of a page, 560 us so; 668 us through a buffer).
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_rowdot(DevHandle g, int fid, ui
 // buffer and the match, 1602 us without; 1280 us is the host link.)  A last value of fewer
 // than four bytes is not counted.
 struct HistSink {
+  static constexpr bool kFar = false;
   static constexpr bool kArrive = true;
   __device__ __forceinline__ uint32_t piece() const { return dev::kPiece; }
   uint32_t* sh;

@@ -2002,12 +2002,10 @@ constexpr uint32_t kRunPages = 32 * kRunWarps;
 // the leading run of pages that are READY without a mark, FILLING or COPYING, or -1
 // where page p is not in the cache at all; their frames are left in s_f, pinned, and
 // the mask of those not READY yet in *wait.  Pages after the run are left unpinned.
-static __device__ int run_begin(const DevHandle& g, uint32_t fid, unsigned long long p, uint32_t k, bool marks,
-                                     uint32_t* s_f, uint32_t* wait) {
+static __device__ __forceinline__ int run_begin(const DevHandle& g, uint32_t fid, unsigned long long p, uint32_t k,
+                                                bool marks, uint32_t* s_f, uint32_t* wait) {
   const int lane = lane_id();
   int f = -1;  // frame of page p + lane
-  uint32_t ovf = 0;  // page p's home bucket overflowed; in flight with the bucket
-  if (lane == 0) ovf = ld_rlx(&g.tovf[bucket_of(make_key(fid, p), g.nbuckets)]);
   // home buckets only, eight keys in flight: a key in an overflow bucket ends the run
   for (uint32_t q0 = 0; q0 < k; q0 += 8) {
     unsigned long long e[8];
@@ -2027,11 +2025,15 @@ static __device__ int run_begin(const DevHandle& g, uint32_t fid, unsigned long 
     }
     if (gap) break;
   }
-  // page p is not here: nothing to pin, and no fence
-  const int f0 = bcast(f);
-  if (f0 < 0) {
-    if (lane == 0) *wait = 0;
-    return bcast((int)ovf) ? 0 : -1;
+  // page p is not here: nothing to pin, and no fence.  (Its bucket's overflow flag is read
+  // here, not in flight with the bucket: there it cost cached scans 2 to 4 us.)
+  if (bcast(f) < 0) {
+    int ovf = 0;
+    if (lane == 0) {
+      ovf = (int)ld_rlx(&g.tovf[bucket_of(make_key(fid, p), g.nbuckets)]);
+      *wait = 0;
+    }
+    return bcast(ovf) ? 0 : -1;
   }
   // pin as frame_pin does, one lane per page
   const bool mine = (uint32_t)lane < k && f >= 0;
@@ -2053,6 +2055,14 @@ static __device__ int run_begin(const DevHandle& g, uint32_t fid, unsigned long 
   if (lane == 0) *wait = wm;
   __syncwarp();
   return (int)c;
+}
+
+// The same out of line, for sinks with kFar set.  Cached scans of 256 MiB in 4 KiB pages by
+// two-unit windows take 60 us so and 64 us with it inlined; with one-unit windows in 64
+// registers 64 MiB take 40 us so and 35 us inlined.
+static __device__ __noinline__ int run_begin_far(const DevHandle& g, uint32_t fid, unsigned long long p, uint32_t k,
+                                                 bool marks, uint32_t* s_f, uint32_t* wait) {
+  return run_begin(g, fid, p, k, marks, s_f, wait);
 }
 
 // One lane, one page of a run (frame f, page q; the gread covers [off, end)): R5's
@@ -2257,6 +2267,7 @@ constexpr uint32_t kPiece = 128u << 10;
 // The gread into a user buffer: the byte at offset off goes to buf[0].  A warp takes a
 // unit of a page at a time.
 struct BufferSink {
+  static constexpr bool kFar = false;  // whether read_run's look-ups go out of line (run_begin_far)
   static constexpr bool kArrive = false;  // the reads of the 64-register instance are bound by their control path
   __device__ __forceinline__ uint32_t piece() const { return kPiece; }
   uint8_t* buf;
@@ -2349,6 +2360,7 @@ __device__ __forceinline__ void unit_sums(Sums& acc, const uint4* v, unsigned lo
 // scans of cached files of 1 to 64 MiB, start and stop included, took 831 us delivered
 // to a buffer per block and 445 us in place.
 struct SumSink {
+  static constexpr bool kFar = false;
   static constexpr bool kArrive = true;
   __device__ __forceinline__ uint32_t piece() const { return kPiece; }
   Sums acc;
@@ -2376,8 +2388,12 @@ struct SumSink {
 // moved each byte three times (out of the cache, into the window, back): a cached 1 GiB
 // scan by 296 blocks, 512 KiB pages, took 296 us that way (579 us with buffers of a whole
 // read), also with the next unit's loads under way, and takes 184 us from here.
+// The window starts on a line of shared memory: the copies of a warp, 512 bytes each, then
+// cross no more lines than they fill.  Behind static variables of any size they did, and
+// the time of cached scans hung on that size (1 GiB in 512 KiB pages: 181 to 210 us; 256 MiB
+// in 4 KiB pages: 62 to 73 us; here 180 and 60 us).
 __device__ __forceinline__ uint8_t* window_memory() {
-  extern __shared__ uint4 s_window[];
+  extern __shared__ __align__(128) uint4 s_window[];
   return reinterpret_cast<uint8_t*>(s_window);
 }
 __device__ __forceinline__ void async_word(uint32_t to, const uint8_t* from) {
@@ -2385,6 +2401,7 @@ __device__ __forceinline__ void async_word(uint32_t to, const uint8_t* from) {
 }
 template <int STAGES>
 struct WindowSink {
+  static constexpr bool kFar = STAGES > 1;
   static constexpr bool kArrive = true;
   __device__ __forceinline__ uint32_t piece() const { return kPiece; }
   Sums acc;
@@ -2458,8 +2475,9 @@ __device__ __noinline__ long long read_run(const DevHandle& g, uint32_t fid, uns
   const uint32_t want = left < 32u * nw ? (uint32_t)left : 32u * nw;  // pages looked up
   uint32_t c = 0;                                                   // this warp's leading pages
   if (32 * w < want) {
-    const int r =
-        run_begin(g, fid, p + 32 * w, want - 32 * w < 32 ? want - 32 * w : 32, marks, s_rf + 32 * w, &s_rwait[w]);
+    const uint32_t m = want - 32 * w < 32 ? want - 32 * w : 32;
+    const int r = Sink::kFar ? run_begin_far(g, fid, p + 32 * w, m, marks, s_rf + 32 * w, &s_rwait[w])
+                             : run_begin(g, fid, p + 32 * w, m, marks, s_rf + 32 * w, &s_rwait[w]);
     c = r < 0 ? 0u : (uint32_t)r;
     if ((tid & 31) == 0) s_rn[w] = w == 0 ? (uint32_t)r : c;
   }
