@@ -158,24 +158,22 @@ struct RowdotSink {
 };
 
 // Block b reads stripes b, b + B, ...; a stripe is `stripe_rows` rows and is read
-// in pieces of `read_len` bytes (whole rows).
+// in pieces of `rows_per_piece` rows.
 __global__ void __launch_bounds__(kThreads, 2) k_rowdot(DevHandle g, int fid, uint32_t rows, uint32_t cols,
                                                      const float* __restrict__ vec, float* __restrict__ out,
-                                                     uint32_t stripe_rows, unsigned long long read_len,
+                                                     uint32_t stripe_rows, uint32_t nstripes, uint32_t rows_per_piece,
                                                      unsigned long long* stripe_sum,
                                                      unsigned long long* stripe_hash, long long* status) {
   __shared__ float4 s_carry[64];
   const unsigned long long row_bytes = (unsigned long long)cols * 4;
-  const uint32_t rows_per_piece = (uint32_t)(read_len / row_bytes);
-  const uint32_t nstripes = (rows + stripe_rows - 1) / stripe_rows;
   RowdotSink sink{reinterpret_cast<const float4*>(vec), out, s_carry, 0ull, row_bytes, cols / 4, 0u, {0ull, 0ull}};
   for (uint32_t st = blockIdx.x; st < nstripes; st += gridDim.x) {
     const uint32_t r0 = st * stripe_rows;
-    const uint32_t r1 = r0 + stripe_rows < rows ? r0 + stripe_rows : rows;
+    const uint32_t r1 = rows - r0 > stripe_rows ? r0 + stripe_rows : rows;
     sink.acc = dev::Sums{0ull, 0ull};
     long long err = 0;
-    for (uint32_t pr = r0; pr < r1; pr += rows_per_piece) {
-      const uint32_t nr = pr + rows_per_piece < r1 ? rows_per_piece : r1 - pr;
+    for (uint32_t pr = r0, nr; pr < r1; pr += nr) {
+      nr = rows_per_piece < r1 - pr ? rows_per_piece : r1 - pr;
       sink.off = (unsigned long long)pr * row_bytes;
       sink.out = out + pr;
       const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, sink.off, nr * row_bytes, sink);
@@ -313,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_histogram(DevHandle g, int fid,
   __shared__ uint32_t sh[kSmemBins];
   for (uint32_t i = threadIdx.x; i < kSmemBins; i += blockDim.x) sh[i] = 0;
   __syncthreads();
-  const unsigned long long npieces = (size + read_len - 1) / read_len;
+  const unsigned long long npieces = size / read_len + (size % read_len != 0);
   HistSink sink{sh, hist, nbins, 0u, 0u, 0ull, {0ull, 0ull}};
   for (unsigned long long pc = blockIdx.x; pc < npieces; pc += gridDim.x) {
     const long long n = dev::gread_impl(g, (int)blockIdx.x, fid, pc * read_len, read_len, sink);
@@ -356,11 +354,13 @@ extern "C" int gfs_rowdot(gfs_ctx* ctx, int fid, uint32_t rows, uint32_t cols, c
   if (rc) return rc;
   note_read(ctx, fid);
   DevHandle g = ctx->dev;
-  g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
-                                      : blocks * (uint32_t)((read_len + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;
+  g.reserve = frame_reserve(ctx, blocks, read_len);
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(d_status, 0, 8, s) != cudaSuccess) return -EINVAL;
-  k_rowdot<<<blocks, kThreads, 0, s>>>(g, fid, rows, cols, d_vec, d_out, stripe_rows, read_len,
+  // a piece ends with its stripe: longer ones would not fit 32 bits, nor would their ends
+  const uint32_t piece = (uint32_t)(read_len / row_bytes < stripe_rows ? read_len / row_bytes : stripe_rows);
+  const uint32_t nstripes = rows / stripe_rows + (rows % stripe_rows != 0);
+  k_rowdot<<<blocks, kThreads, 0, s>>>(g, fid, rows, cols, d_vec, d_out, stripe_rows, nstripes, piece,
                                        (unsigned long long*)d_stripe_sum, (unsigned long long*)d_stripe_hash, (long long*)d_status);
   return cudaGetLastError() == cudaSuccess ? 0 : -EINVAL;
 }
@@ -375,8 +375,7 @@ extern "C" int gfs_histogram(gfs_ctx* ctx, int fid, uint32_t nbins, uint32_t* d_
   if (rc) return rc;
   note_read(ctx, fid);
   DevHandle g = ctx->dev;
-  g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
-                                      : blocks * (uint32_t)((read_len + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;
+  g.reserve = frame_reserve(ctx, blocks, read_len);
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(d_hist, 0, (size_t)nbins * 4, s) != cudaSuccess) return -EINVAL;
   if (cudaMemsetAsync(d_sums, 0, 16, s) != cudaSuccess) return -EINVAL;

@@ -1246,10 +1246,7 @@ static int scan_prepare(gfs_ctx* ctx, int fid, const gfs_scan_args* a, uint64_t*
   }
   *g = ctx->dev;
   g->exact_lra = a->serialize ? 1u : 0u;
-  const uint64_t pages_per_read = (a->read_len >> ctx->dev.page_shift) + ((a->read_len & (ctx->cfg.page_size - 1)) != 0);
-  g->reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
-                                       : (uint32_t)(pages_per_read >= 0xffffffffull / a->blocks ? 0xffffffffull
-                                                                      : a->blocks * pages_per_read + 1);
+  g->reserve = frame_reserve(ctx, a->blocks, a->read_len);
   if (a->serialize) {
     int maxb = 0;
     int rc = scan_max_resident_blocks(a->threads, ctx->cfg.device, &maxb);
@@ -1295,10 +1292,7 @@ int gfs_scan_path(gfs_ctx* ctx, const char* path, const gfs_scan_args* a, int64_
   const int rc = ensure_paper_state(ctx, a->blocks);
   if (rc) return rc;
   DevHandle g = ctx->dev;
-  const uint64_t pages_per_read = (a->read_len >> ctx->dev.page_shift) + ((a->read_len & (ctx->cfg.page_size - 1)) != 0);
-  g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
-                                      : (uint32_t)(pages_per_read >= 0xffffffffull / a->blocks ? 0xffffffffull
-                                                                      : a->blocks * pages_per_read + 1);
+  g.reserve = frame_reserve(ctx, a->blocks, a->read_len);
   PathArg pa;
   memset(pa.s, 0, sizeof(pa.s));
   memcpy(pa.s, path, len);
@@ -1310,10 +1304,7 @@ int gfs_device_handle(gfs_ctx* ctx, uint32_t blocks, uint64_t read_len, void* ou
   if (cap < sizeof(DevHandle)) return -ENOSPC;
   __atomic_store_n(&ctx->handle_out, (uint8_t)1, __ATOMIC_RELAXED);
   DevHandle g = ctx->dev;
-  const uint64_t pages_per_read = (read_len >> ctx->dev.page_shift) + ((read_len & (ctx->cfg.page_size - 1)) != 0);
-  g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
-                                      : (uint32_t)(pages_per_read >= 0xffffffffull / blocks ? 0xffffffffull
-                                                                      : blocks * pages_per_read + 1);
+  g.reserve = frame_reserve(ctx, blocks, read_len);
   memcpy(out, &g, sizeof(g));
   return (int)sizeof(DevHandle);
 }

@@ -112,6 +112,15 @@ struct gfs_ctx {
   std::mutex dev_open_mu;          // device opens and closes, one at a time
 };
 
+// The frames that readahead leaves alone for greads of read_len bytes by `blocks` blocks:
+// the configured reserve, or all pages they touch at once and one more (saturating).
+inline uint32_t frame_reserve(const gfs_ctx* ctx, uint32_t blocks, uint64_t read_len) {
+  if (ctx->cfg.reserve_frames) return ctx->cfg.reserve_frames;
+  const uint64_t pages = (read_len >> ctx->dev.page_shift) + ((read_len & (ctx->cfg.page_size - 1)) != 0);
+  if (pages >= 0xffffffffull / blocks) return 0xffffffffu;
+  return (uint32_t)(blocks * pages + 1);
+}
+
 // Call when launching a kernel that reads fid.  Returns whether none of the file's pages
 // can be cached yet (no such launch since they were last dropped).
 inline bool note_read(gfs_ctx* ctx, int fid) {

@@ -275,11 +275,7 @@ extern "C" int gfs_scan_static(gfs_ctx* ctx, int fid, const gfs_scan_args* a, in
   note_read(ctx, fid);
   gfs::DevHandle g = ctx->dev;
   g.exact_lra = a->serialize ? 1u : 0u;
-  const uint64_t pages_per_read = (a->read_len >> ctx->dev.page_shift) + ((a->read_len & (ctx->cfg.page_size - 1)) != 0);
-  g.reserve = ctx->cfg.reserve_frames
-                  ? ctx->cfg.reserve_frames
-                  : (uint32_t)(pages_per_read >= 0xffffffffull / a->blocks ? 0xffffffffull
-                                                                             : (uint64_t)a->blocks * pages_per_read + 1);
+  g.reserve = frame_reserve(ctx, a->blocks, a->read_len);
   cudaStream_t s = (cudaStream_t)stream;
   if (a->serialize) {
     int maxb = 0;

@@ -138,7 +138,7 @@ __device__ void admit(const DevHandle& g, const Handle& h) {
     SubSlot* ss = &h.sub[t % h.sub_slots];
     if (dev::ld_acq_sys64(&ss->seq) != t + 1) return;  // nothing waiting
     const unsigned long long len = ss->len;
-    const uint32_t n_units = (uint32_t)((len + h.unit_bytes - 1) / h.unit_bytes);
+    const uint32_t n_units = (uint32_t)(len / h.unit_bytes + (len % h.unit_bytes != 0));
     const uint32_t cap = n_units < h.units_cap ? n_units : h.units_cap;
     const uint32_t frames = cap * h.pages_per_unit;
     const unsigned long long reserved = dev::ld_rlx64(&h.ctl->frames_reserved.v);
@@ -374,7 +374,9 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   h.max_req = sc->max_requests;
   h.unit_bytes = sc->unit_bytes;
   h.units_cap = sc->units_in_flight ? sc->units_in_flight : 16;
-  h.pages_per_unit = (uint32_t)((sc->unit_bytes + ctx->cfg.page_size - 1) / ctx->cfg.page_size) + 1;
+  // more pages than there can be frames are reserved as that many
+  const uint64_t unit_pages = sc->unit_bytes / ctx->cfg.page_size + (sc->unit_bytes % ctx->cfg.page_size != 0) + 1;
+  h.pages_per_unit = unit_pages < MAX_FRAMES ? (uint32_t)unit_pages : (uint32_t)MAX_FRAMES;
   const uint32_t F = ctx->dev.n_frames;
   const uint64_t in_use = (uint64_t)sc->ctas * h.pages_per_unit;
   h.frame_budget = sc->frame_budget ? sc->frame_budget : (uint32_t)(F > in_use ? F - in_use : F / 2);
@@ -426,7 +428,8 @@ extern "C" int gfs_serve_start(gfs_ctx* ctx, const gfs_serve_config* sc, void* s
   h.ctl = (Ctl*)(s->d_mem + ctl_off);
   s->h = h;
   DevHandle g = ctx->dev;
-  g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames : (uint32_t)(in_use + 1);
+  g.reserve = ctx->cfg.reserve_frames ? ctx->cfg.reserve_frames
+                                      : (in_use < 0xffffffffull ? (uint32_t)(in_use + 1) : 0xffffffffu);
   if ((int)sc->ctas <= per_sm_wide * sms) k_serve<1><<<sc->ctas, sc->threads, 0, s->stream>>>(g, h);
   else k_serve<2><<<sc->ctas, sc->threads, 0, s->stream>>>(g, h);
   rc = cerr(cudaGetLastError());
