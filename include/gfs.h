@@ -331,7 +331,9 @@ int gfs_scan_host(gfs_ctx* ctx, int fid, const gfs_scan_args* args, int64_t* h_c
  * read in shared memory.
  *   - blocks * round_up(min(read_len, file size), 256) must fit in
  *     GFS_STATIC_SCRATCH_BYTES, else the call returns -ENOSPC and launches
- *     nothing.
+ *     nothing.  (The bound dates from when the blocks had buffers in device
+ *     memory; it stays part of the interface, as does gfs_scan's -ENOMEM for a
+ *     product that overflows size_t.)
  *   - With GFS_MODE_PAPER or GFS_REPL_TB_LRA the context keeps per-threadblock
  *     state that an allocating call sizes: -ENOTSUP until a gfs_scan (or
  *     gfs_scan_path, gfs_read_many) with at least `blocks` threadblocks has run
@@ -435,7 +437,10 @@ int gfs_serve_stop(gfs_ctx* ctx);
  * greads each stripe in pieces of read_len bytes (a multiple of the row size);
  * d_out[r] = sum_c A[r][c] * d_vec[c] in float32 (FMA, any summation order);
  * d_stripe_sum / d_stripe_hash[s] = the byte checksums of stripe s (as in
- * gfs_scan); *d_status = 0 or the first -errno.  d_vec holds cols floats. */
+ * gfs_scan); *d_status = 0 or the first -errno.  d_vec holds cols floats.  Rows are
+ * taken from the cache as their pages come in, so a call that fails half way may have
+ * written rows of the piece that failed, and its stripe's checksums cover the bytes taken
+ * until then. */
 int gfs_rowdot(gfs_ctx* ctx, int fid, uint32_t rows, uint32_t cols, const float* d_vec, float* d_out,
                uint32_t stripe_rows, uint64_t read_len, uint32_t blocks, uint64_t* d_stripe_sum,
                uint64_t* d_stripe_hash, int64_t* d_status, void* stream);
@@ -443,7 +448,9 @@ int gfs_rowdot(gfs_ctx* ctx, int fid, uint32_t rows, uint32_t cols, const float*
 /* gfs_histogram: file fid holds int32 values; d_hist[nbins] (zeroed by the call)
  * receives the count of each value v < nbins; d_sums[0] = sum of all bytes read
  * mod 2^64, d_sums[1] = values >= nbins; *d_status = 0 or the first -errno.
- * Block b greads pieces b, b+blocks, ... of read_len bytes (a multiple of 16). */
+ * Block b greads pieces b, b+blocks, ... of read_len bytes (a multiple of 16).  After a
+ * failure (*d_status < 0) d_hist and d_sums hold what was counted until then, part of the
+ * failing piece included. */
 int gfs_histogram(gfs_ctx* ctx, int fid, uint32_t nbins, uint32_t* d_hist, uint64_t read_len, uint32_t blocks,
                   uint64_t* d_sums, int64_t* d_status, void* stream);
 

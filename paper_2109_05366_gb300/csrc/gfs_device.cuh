@@ -2387,7 +2387,7 @@ struct SumSink {
 // Bound by HBM reads.  A window in device memory that stayed in L2 was bound by L2, which
 // moved each byte three times (out of the cache, into the window, back): a cached 1 GiB
 // scan by 296 blocks, 512 KiB pages, took 296 us that way (579 us with buffers of a whole
-// read), also with the next unit's loads under way, and takes 184 us from here.
+// read), also with the next unit's loads under way, and takes 180 us from here.
 // The window starts on a line of shared memory: the copies of a warp, 512 bytes each, then
 // cross no more lines than they fill.  Behind static variables of any size they did, and
 // the time of cached scans hung on that size (1 GiB in 512 KiB pages: 181 to 210 us; 256 MiB

@@ -41,8 +41,8 @@ struct HostFile {
   // closed on the device: the id keeps its cached pages (and its descriptor)
   // until they are dropped at a quiet point
   bool retired = false;
-  // a kernel that may bring pages of the file into the cache was launched since they
-  // were last dropped (relaxed atomic access; only picks a kernel instance)
+  // a kernel that may bring pages of the file into the cache was launched since the last
+  // gfs_reset_cache (relaxed atomic access; only picks a kernel instance)
   uint8_t maybe_cached = 0;
 };
 
@@ -122,7 +122,7 @@ inline uint32_t frame_reserve(const gfs_ctx* ctx, uint32_t blocks, uint64_t read
 }
 
 // Call when launching a kernel that reads fid.  Returns whether none of the file's pages
-// can be cached yet (no such launch since they were last dropped).
+// can be cached yet (no such launch since the last gfs_reset_cache).
 inline bool note_read(gfs_ctx* ctx, int fid) {
   gfs::HostFile& f = ctx->files[fid];
   return !__atomic_exchange_n(&f.maybe_cached, (uint8_t)1, __ATOMIC_RELAXED) && !f.by_device &&

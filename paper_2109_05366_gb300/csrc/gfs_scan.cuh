@@ -60,14 +60,15 @@ static __device__ void block_help_drain(const DevHandle& g) {
     if (!dev::block_help(g, -1, true)) break;
 }
 
+// A warp's window: two units, or one where four blocks of 256 threads share an SM (their
+// windows are then as large together, and the other blocks' warps cover a warp's waits).
+__host__ __device__ constexpr int scan_stages(int minb) { return minb == 1 ? 2 : 1; }
+inline size_t scan_window(int minb, uint32_t threads) { return (size_t)scan_stages(minb) * (threads / 32) * 4096; }
+
 // MAXT, MINB: the largest block the instance is compiled for and the blocks per
 // SM it must leave room for, which set its register budget.  <512, 1> leaves the
 // control path every register it uses (no spills; two 256-thread blocks per SM);
 // <256, 4> fits four 256-thread blocks per SM in 64 registers.
-// A warp's window: two units, or one where four blocks of 256 threads share an SM.
-__host__ __device__ constexpr int scan_stages(int minb) { return minb == 1 ? 2 : 1; }
-inline size_t scan_window(int minb, uint32_t threads) { return (size_t)scan_stages(minb) * (threads / 32) * 4096; }
-
 template <int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsigned long long stride,
                                                unsigned long long read_len, unsigned long long nstrides, int serialize,
@@ -109,7 +110,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_scan(DevHandle g, int fid, unsig
 // Independent greads (Section 2.2): block b serves reads b, b + B, ... of the
 // list.  MAXT, MINB as for k_scan: a small read costs a block mostly control-path
 // latency, so the reads in flight grow with the blocks resident per SM.
-// BATCH: reads of cached pages go in batches.  Both instances also exist without, for lists on files of which nothing can be cached yet: there the batches' call makes the
+// BATCH: reads of cached pages go in batches.  Both instances also exist without, for
+// lists on files of which nothing can be cached yet: there the batches' call makes the
 // register allocator spill what gread holds (131072 random 4 KiB pages from the host:
 // 2337 us with, 2223 us without).
 template <bool BATCH, int MAXT, int MINB>
